@@ -73,7 +73,7 @@ def kernel_label(t):
     if t[0] > 0:
         return "cluster-resident, %d CTAs per solve" % t[0]
     if t[0] == -2:
-        return "two-step TMA streaming (two leap-frog steps per pass, persistent, 4-stage mbarrier ring)"
+        return "multi-step streaming (four leap-frog steps per pass over column strips, cp.async ring)"
     if t[0] < 0:
         return "TMA streaming (persistent, 4-stage mbarrier ring)"
     return "streaming, %d rows/thread, %d warps/block" % (t[1], t[2])
@@ -162,12 +162,11 @@ def measured_peaks():
 KERNEL_SOURCES = {"k_resident": ("resident.cu", "pair_math.cuh", "stencil_cell.cuh", "oed_internal.cuh"),
                   "k_step": ("stencil.cu", "stencil_cell.cuh", "oed_internal.cuh"),
                   "k_step_tma": ("stream_tma.cu", "tma_sync.cuh", "stencil_cell.cuh", "oed_internal.cuh"),
-                  "k_step2_tma": ("stream_tma2.cu", "pair_math.cuh", "tma_sync.cuh", "stencil_cell.cuh",
-                                  "oed_internal.cuh")}
+                  "k_strip": ("stream_strip.cu", "pair_math.cuh", "stencil_cell.cuh", "oed_internal.cuh")}
 
 
 def streaming_kernel_name(tuning) -> str:
-    return {-2: "k_step2_tma", -1: "k_step_tma"}.get(tuning[0], "k_step")
+    return {-2: "k_strip", -1: "k_step_tma"}.get(tuning[0], "k_step")
 
 
 def _code_only(text: str) -> str:
@@ -621,7 +620,7 @@ def measure_layered(P, torch, dev, args, rank, oracle_nodes=2):
     n = x.shape[0]
     # the rule lists its nodes grouped by the coordinates they vary (in some runs of 96
     # nodes every source sits at one position); taking every k-th node per chunk spreads
-    # each chunk's sources over the grid, which the two-step kernel runs faster (the sum
+    # each chunk's sources over the grid, as a Monte Carlo batch has them (the sum
     # does not depend on the order)
     nchunk = (n + chunk_nodes - 1) // chunk_nodes
     perm = np.concatenate([np.arange(c, n, nchunk) for c in range(nchunk)])

@@ -85,13 +85,13 @@ static Sizes sizes(const Geometry &g, int precision, int max_solves)
     const int chunk = std::max(1, max_solves / kND);   // the larger of the two node chunks
     Sizes s;
     auto al = [](size_t b) { return (b + 255) / 256 * 256; };
-    // FP32 grids that do not fit on chip keep a second pair of levels for the two-step
-    // kernel (it reads one pair and writes the other), whose paired layout may need a
+    // FP32 grids that do not fit on chip keep a second pair of levels for the multi-step
+    // kernel (it reads one pair and writes the other), whose strip layout may need a
     // little more than the planar one per solve
-    const bool two_step = precision == OED_FP32 && !resident_fits(g);
-    const size_t per = two_step ? std::max(g.solve_stride, paired_stride(g)) : g.solve_stride;
+    const bool multi_step = precision == OED_FP32 && !resident_fits(g);
+    const size_t per = multi_step ? std::max(g.solve_stride, strip_stride(g)) : g.solve_stride;
     s.u = al((size_t)max_solves * per * e);
-    s.u2 = two_step ? 2 * s.u : 0;
+    s.u2 = multi_step ? 2 * s.u : 0;
     s.kp = s.u2 ? al((size_t)g.nz * 16 * sizeof(float)) : 0;   // packed row coefficients
     s.src = al((size_t)max_solves * (precision == OED_FP64 ? sizeof(SourceDesc<double>)
                                                            : sizeof(SourceDesc<float>)));
@@ -413,18 +413,15 @@ int oed_autotune(oed_ctx *ctx, int nsolve, void *stream)
             best = ctx->tune;
         }
     }
-    // two-step TMA streaming kernel (FP32 grids that do not fit on chip).  It is taken
-    // whenever it runs: short probes time it well below its rate in a real time loop
-    // (801x401, 1792 solves: 211 Gcell-upd/s in a 16- or 64-step probe, on zero, random
-    // or smooth data alike, against 304 in a 1200-step solve, where the one-step kernel
-    // probes and runs at 230), so the probe only checks that it launches.
-    if (ctx->d_u2 && tma_supported(ctx) && tma_prepare(ctx) > 0 && tma2_prepare(ctx) > 0) {
+    // multi-step strip kernel (FP32 grids that do not fit on chip).  It is taken whenever it
+    // runs: it moves a third of the one-step kernels' bytes per step (801x401, three layers,
+    // 672 solves: 705 Gcell-upd/s against 247), so the probe only checks that it launches.
+    if (ctx->d_u2 && strip_prepare(ctx) > 0) {
         ctx->tune = StepTuning{best.zs, best.wz, -2};
         int probe = std::min(ctx->g.nsteps, std::max(nrep, 16));
         probe = probe < 4 ? probe : probe / 2 * 2;
-        const float *last = nullptr;
-        cudaError_t e = launch_steps_tma2(ctx, nsolve, st, e0, e1, 2, &last);   // warm
-        if (e == cudaSuccess) e = launch_steps_tma2(ctx, nsolve, st, e0, e1, probe, &last);
+        cudaError_t e = launch_steps_strip(ctx, nsolve, st, e0, e1, 4);   // warm
+        if (e == cudaSuccess) e = launch_steps_strip(ctx, nsolve, st, e0, e1, probe);
         if (e == cudaSuccess) e = cudaEventSynchronize(e1);
         float ms = 0.0f;
         if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
@@ -494,9 +491,9 @@ int oed_set_tuning(oed_ctx *ctx, int cluster_size, int rows_per_thread, int warp
         if (!tma_supported(ctx) || tma_prepare(ctx) < 1)
             return set_err(ctx, OED_EINVAL, "oed_set_tuning: the TMA kernel needs FP32");
     } else if (cluster_size == -2) {
-        if (!ctx->d_u2 || !tma_supported(ctx) || tma_prepare(ctx) < 1 || tma2_prepare(ctx) < 1)
+        if (!ctx->d_u2 || strip_prepare(ctx) < 1)
             return set_err(ctx, OED_EINVAL,
-                           "oed_set_tuning: the two-step TMA kernel needs FP32 and a grid that does not fit on chip");
+                           "oed_set_tuning: the multi-step kernel needs FP32 and a grid that does not fit on chip");
     } else if (cluster_size != 0) {
         const int cmin = resident_cluster_size(ctx);
         if (cmin == 0 || cluster_size < cmin || cluster_size > 8 ||

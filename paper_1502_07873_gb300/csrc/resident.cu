@@ -48,7 +48,6 @@ namespace oed {
 // two, four or five.
 constexpr int kResThreads = 640;
 constexpr int kResRegs = 96;
-constexpr bool kPS = true;   // the packed-subtract form of the pair arithmetic
 
 struct ResArgs {
     const FacCoef<float> *fac;     // [nz]
@@ -128,7 +127,7 @@ __device__ __forceinline__ void pair_put_n(float2 *q, int offE, int offO, float4
 
 __device__ __forceinline__ void load_row(const float2 *q, int sq, Row2P &r)
 {
-    row_fromP<kPS>(q[sq - 1], pair_at(q, sq), q[1], r);
+    row_fromP(q[sq - 1], pair_at(q, sq), q[1], r);
 }
 
 // the same slots of a row in CTA `nb` of the cluster
@@ -143,7 +142,7 @@ __device__ __forceinline__ void load_row_remote(const float2 *q, int sq, unsigne
 {
     const unsigned b = remote_addr(smem_addr(q), nb);
     const float2 e = ld_cluster2(b), o = ld_cluster2(b + 8u * (unsigned)sq);
-    row_fromP<kPS>(ld_cluster2(b + 8u * (unsigned)(sq - 1)), make_float4(e.x, e.y, o.x, o.y), ld_cluster2(b + 8u), r);
+    row_fromP(ld_cluster2(b + 8u * (unsigned)(sq - 1)), make_float4(e.x, e.y, o.x, o.y), ld_cluster2(b + 8u), r);
 }
 
 // float offset of node (column i, component comp) within a shared row
@@ -249,13 +248,13 @@ __global__ void __maxnreg__(kResRegs) k_resident(ResArgs a)
                     load_row(cur + (l + 1) * RS, sq, rs);
                 else   // a one-row slab
                     load_row_remote(cur, sq, rank + 1, rs);
-                southP<kPS>(rc, rs);
+                southP(rc, rs);
                 Row2P nt = rc;
                 nt.va = nt.vb = make_float2(0.0f, 0.0f);
                 float2 *o = nxt + l * RS;
                 float4 u = pair_at_n(o, offE, offO);
                 const KP K = coef[l];
-                pair_updateP<kPS>(K, nt, rc, rs, u);
+                pair_updateP(K, nt, rc, rs, u);
                 pair_put_n(o, offE, offO, u);
                 rn = rc;
                 rc = rs;
@@ -265,7 +264,7 @@ __global__ void __maxnreg__(kResRegs) k_resident(ResArgs a)
                     load_row(cur + (l - 1) * RS, sq, rn);
                 else
                     load_row_remote(cur + (R - 1) * RS, sq, rank - 1, rn);
-                southP<kPS>(rn, rc);
+                southP(rn, rc);
             }
             // rows whose south neighbour is a local row and that are not the bottom row:
             // unrolled by three with the three window rows taking turns
@@ -282,7 +281,7 @@ __global__ void __maxnreg__(kResRegs) k_resident(ResArgs a)
                 // unifK: the CTA's march rows share K0 (no coefficient loads)
                 auto march = [&](auto unifK) {
                     auto row = [&](auto pf, const Row2P &wn, Row2P &wc, Row2P &ws) {
-                        row_fromP<kPS>(pw, pm, pe, ws);
+                        row_fromP(pw, pm, pe, ws);
                         float4 u = pu;
                         if constexpr (decltype(pf)::value) {
                             sp += RS;
@@ -291,9 +290,9 @@ __global__ void __maxnreg__(kResRegs) k_resident(ResArgs a)
                             pe = sp[1];
                             pu = pair_at_n(o + RS, offE, offO);
                         }
-                        southP<kPS>(wc, ws);
+                        southP(wc, ws);
                         const KP K = decltype(unifK)::value ? K0 : *cf;
-                        pair_updateP<kPS>(K, wn, wc, ws, u);
+                        pair_updateP(K, wn, wc, ws, u);
                         pair_put_n(o, offE, offO, u);
                         o += RS;
                         cf++;
@@ -344,8 +343,8 @@ __global__ void __maxnreg__(kResRegs) k_resident(ResArgs a)
                     absorbingP(K.c, nv, rc, true, 0, u);
                 } else {
                     load_row_remote(cur, sq, rank + 1, rs);
-                    southP<kPS>(rc, rs);
-                    pair_updateP<kPS>(K, rn, rc, rs, u);
+                    southP(rc, rs);
+                    pair_updateP(K, rn, rc, rs, u);
                 }
                 pair_put_n(o, offE, offO, u);
                 rn = rc;

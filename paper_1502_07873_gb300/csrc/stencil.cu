@@ -227,7 +227,7 @@ __global__ void k_fill_probe(real *__restrict__ u, size_t n, unsigned salt)
 void launch_fill_probe(const oed_ctx *ctx, int nsolve, cudaStream_t st)
 {
     size_t per = ctx->g.solve_stride;
-    if (ctx->d_u2) per = per > paired_stride(ctx->g) ? per : paired_stride(ctx->g);
+    if (ctx->d_u2) per = per > strip_stride(ctx->g) ? per : strip_stride(ctx->g);
     const size_t n = (size_t)nsolve * per;
     void *lv[4] = {ctx->d_u0, ctx->d_u1, ctx->d_u2, ctx->d_u3};
     for (int k = 0; k < 4; k++) {
@@ -253,17 +253,11 @@ void launch_step_probe(const oed_ctx *ctx, int nsolve, int nrep, cudaStream_t st
 cudaError_t launch_forward_steps(const oed_ctx *ctx, int nsolve, cudaStream_t st, cudaEvent_t ev0,
                                  cudaEvent_t ev1)
 {
-    if (ctx->tune.C == -2) {   // the two-step kernel's paired layout
-        const size_t pb = (size_t)nsolve * paired_stride(ctx->g) * sizeof(float);
+    if (ctx->tune.C == -2) {   // the multi-step kernel's strip layout
+        const size_t pb = 2 * (size_t)nsolve * strip_stride(ctx->g) * sizeof(float);
         cudaMemsetAsync(ctx->d_u0, 0, pb, st);
-        cudaMemsetAsync(ctx->d_u1, 0, pb, st);
         cudaMemsetAsync(ctx->d_u2, 0, pb, st);
-        cudaMemsetAsync(ctx->d_u3, 0, pb, st);
-        const float *last = nullptr;
-        const cudaError_t e = launch_steps_tma2(ctx, nsolve, st, ev0, ev1, 0, &last);
-        if (e != cudaSuccess) return e;
-        launch_tma2_gather(ctx, nsolve, last, ctx->g.nsteps, st);
-        return cudaGetLastError();
+        return launch_steps_strip(ctx, nsolve, st, ev0, ev1, 0);
     }
     const size_t bytes = (size_t)nsolve * ctx->g.solve_stride * ctx->elem;
     cudaMemsetAsync(ctx->d_u0, 0, bytes, st);

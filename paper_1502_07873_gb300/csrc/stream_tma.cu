@@ -271,20 +271,6 @@ bool tma_make_map(CUtensorMap *map, void *base, const Geometry &g, int nsolve, i
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-bool tma_make_paired_map(CUtensorMap *map, void *base, const Geometry &g, int nsolve, int bslots, int bz)
-{
-    auto fn = encode_fn();
-    if (!fn) return false;
-    const int sq = paired_sq(g);
-    const cuuint64_t dims[4] = {(cuuint64_t)(2 * sq), 2, (cuuint64_t)g.nz, (cuuint64_t)nsolve};
-    const cuuint64_t strides[3] = {(cuuint64_t)sq * 8, (cuuint64_t)sq * 16, (cuuint64_t)paired_stride(g) * 4};
-    const cuuint32_t box[4] = {(cuuint32_t)(2 * bslots), 2, (cuuint32_t)bz, 1};
-    const cuuint32_t es[4] = {1, 1, 1, 1};
-    return fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, base, dims, strides, box, es,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 cudaError_t launch_wait_selftest(const oed_ctx *ctx, unsigned long long limit_ns, cudaStream_t st)
 {
     k_wait_selftest<<<1, 32, 0, st>>>(ctx->d_err, limit_ns);
@@ -337,25 +323,6 @@ static void tma_args(const oed_ctx *ctx, int nsolve, TmaArgs &a)
     a.nsolve = nsolve;
     a.nbx = (ctx->g.nx + kTX - 1) / kTX;
     a.nbz = (ctx->g.nz + kTZ - 1) / kTZ;
-}
-
-// One step m of nsolve solves with the one-step kernel on explicit levels: u^m in cur,
-// u^{m-1} in nxt, overwritten with u^{m+1}.
-cudaError_t launch_tma_one_step(const oed_ctx *ctx, int nsolve, cudaStream_t st, float *cur, float *nxt, int m)
-{
-    CUtensorMap halo, plain;
-    if (!tma_make_map(&halo, cur, ctx->g, nsolve, kWX, kWZ) || !tma_make_map(&plain, nxt, ctx->g, nsolve, kTX, kTZ))
-        return cudaErrorInvalidValue;
-    if (ctx->tma_ctas < 1) return cudaErrorInvalidConfiguration;
-    TmaArgs a;
-    tma_args(ctx, nsolve, a);
-    const long long ntile = (long long)nsolve * a.nbx * a.nbz;
-    if (ntile >= (1LL << 31) - 2LL * ctx->tma_ctas) return cudaErrorInvalidValue;
-    const int grid = (int)(ntile < (long long)ctx->tma_ctas ? ntile : (long long)ctx->tma_ctas);
-    a.nxt = nxt;
-    a.m = m;
-    k_step_tma<<<grid, 32 * (kConsumerWarps + 1), kSmemBytes, st>>>(a, halo, plain);
-    return cudaGetLastError();
 }
 
 // All steps of nsolve solves with the TMA kernel (the caller zeroes the levels).
