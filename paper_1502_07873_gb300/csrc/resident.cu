@@ -48,6 +48,8 @@ namespace oed {
 // two, four or five.
 constexpr int kResThreads = 640;
 constexpr int kResRegs = 96;
+constexpr int kResRegsHom = 88;   // homogeneous medium, several CTAs: 640 Gcell-upd/s on 401x201 (96: 629)
+constexpr size_t kSmemPerSm = 228 * 1024;   // shared memory of an SM, 1 KB of it reserved per CTA
 
 struct ResArgs {
     const FacCoef<float> *fac;     // [nz]
@@ -151,11 +153,14 @@ __device__ __forceinline__ int node_off(int i, int comp, int sq)
     return 2 * ((i & 1) ? sq + (i >> 1) + 1 : (i >> 1) + 1) + comp;
 }
 
-__global__ void __maxnreg__(kResRegs) k_resident(ResArgs a)
+// HOM: the medium is homogeneous, so every march row has the coefficients of row 1.
+// ONE: clusters of one CTA, no remote rows and a CTA barrier in place of the cluster's.
+template <bool HOM, bool ONE>
+__global__ void __maxnreg__(HOM && !ONE ? kResRegsHom : kResRegs) k_resident(ResArgs a)
 {
     extern __shared__ float4 smem4[];
     const Geometry &g = a.g;
-    const unsigned rank = cluster_rank();
+    const unsigned rank = ONE ? 0 : cluster_rank();
     const int s = blockIdx.y;
     const int R = a.R, sq = a.sq;
     const int j0 = (int)rank * R;
@@ -203,17 +208,22 @@ __global__ void __maxnreg__(kResRegs) k_resident(ResArgs a)
     const bool patch = active && (scolA || scolB) && sj + kPatch > j0 + l0 && sj < j0 + l1;
     const bool patch_warp = __any_sync(0xffffffffu, patch);
     float *trace = a.trace + (size_t)s * g.nlev * g.nrec * 2;
-    // when every row the march visits in this CTA (rows 1 or 0 .. nrows-2: the surface and
-    // the last row are peeled) has the coefficients of the first, as in a homogeneous
-    // medium, the march keeps them in registers instead of reloading them row by row
-    const int kfirst = (j0 == 0) ? 1 : 0;
+    // The march keeps its rows' coefficients in registers instead of reloading them row by
+    // row: in a homogeneous medium they are the CTA's, otherwise where the march rows of every
+    // lane of a warp (its segment's, without the surface row and the slab's last row, which are
+    // peeled) have one set each, as anywhere but around a layer interface.
+    const int lfirst = HOM ? (j0 == 0 ? 1 : 0) : l0 + (top ? 1 : 0), llast = min(l1, nrows - 1);
     __syncthreads();
-    bool same = true;
-    for (int k = kfirst + 1 + tid; k < nrows - 1; k += nthr) same &= kp_equal(coef[k], coef[kfirst]);
-    const bool unif = __syncthreads_and(same) != 0 && kfirst < nrows - 1;
-    const KP K0 = coef[min(kfirst, nrows - 1)];
+    const KP K0 = coef[min(lfirst, nrows - 1)];
+    bool unif = true;
+    if (!HOM) {
+        bool same = true;
+        if (active)
+            for (int k = lfirst + 1; k < llast; k++) same &= kp_equal(coef[k], K0);
+        unif = __all_sync(0xffffffffu, same) != 0;
+    }
     const int npw = __syncthreads_count(patch_warp && (tid & 31) == 0);
-    cluster_barrier();
+    if (!ONE) cluster_barrier();
 
     for (int m = 0; m < g.nsteps; m++) {
         const float2 *cur = ((m & 1) ? B : A) + p + 1;   // this thread's even slot in row 0
@@ -244,7 +254,7 @@ __global__ void __maxnreg__(kResRegs) k_resident(ResArgs a)
             int l = l0;
             load_row(cur + l * RS, sq, rc);
             if (top) {   // surface row: no north differences, cross terms on the row itself
-                if (l + 1 < nrows)
+                if (ONE || l + 1 < nrows)
                     load_row(cur + (l + 1) * RS, sq, rs);
                 else   // a one-row slab
                     load_row_remote(cur, sq, rank + 1, rs);
@@ -260,7 +270,7 @@ __global__ void __maxnreg__(kResRegs) k_resident(ResArgs a)
                 rc = rs;
                 l++;
             } else {
-                if (l > 0)
+                if (ONE || l > 0)
                     load_row(cur + (l - 1) * RS, sq, rn);
                 else
                     load_row_remote(cur + (R - 1) * RS, sq, rank - 1, rn);
@@ -278,7 +288,7 @@ __global__ void __maxnreg__(kResRegs) k_resident(ResArgs a)
                 float2 pw = sp[sq - 1];
                 float2 pe = sp[1];
                 // pf: a row below the south row exists, prefetch it (every row but the last)
-                // unifK: the CTA's march rows share K0 (no coefficient loads)
+                // unifK: each lane's march rows share its K0 (no coefficient loads)
                 auto march = [&](auto unifK) {
                     auto row = [&](auto pf, const Row2P &wn, Row2P &wc, Row2P &ws) {
                         row_fromP(pw, pm, pe, ws);
@@ -324,9 +334,9 @@ __global__ void __maxnreg__(kResRegs) k_resident(ResArgs a)
                     }
                     l = lstop;
                 };
-                // a CTA-uniform choice: a branch inside the march body would split the
+                // a warp-uniform choice: a branch inside the march body would split the
                 // unrolled rows into separate blocks and cost the scheduler its overlap
-                if (unif)
+                if (HOM || unif)
                     march(std::true_type{});
                 else
                     march(std::false_type{});
@@ -337,8 +347,8 @@ __global__ void __maxnreg__(kResRegs) k_resident(ResArgs a)
                 const KP K = coef[l];
                 float2 *o = nxt + l * RS;
                 float4 u = pair_at_n(o, offE, offO);
-                if (j0 + l == g.nz - 1) {
-                    const float4 nv = l > 0 ? pair_at(cur + (l - 1) * RS, sq)
+                if (ONE || j0 + l == g.nz - 1) {
+                    const float4 nv = ONE || l > 0 ? pair_at(cur + (l - 1) * RS, sq)
                                             : pair_at_remote(cur + (R - 1) * RS, sq, rank - 1);
                     absorbingP(K.c, nv, rc, true, 0, u);
                 } else {
@@ -369,7 +379,10 @@ __global__ void __maxnreg__(kResRegs) k_resident(ResArgs a)
                 row[o + 1] = add_force(row[o + 1], S, sw[kPatch * kPatch + k]);
             }
         }
-        cluster_barrier();
+        if (ONE)
+            __syncthreads();
+        else
+            cluster_barrier();
     }
     if (rank == 0) {
         const float *row0 = reinterpret_cast<const float *>((g.nsteps & 1) ? B : A);
@@ -385,7 +398,17 @@ struct ResShape {
     size_t smem;
 };
 
-static ResShape resident_shape(const Geometry &g, int C)
+// kmax: the most CTAs one SM gets of the launch, so the most that are worth planning for.
+//
+// Small slabs leave room for several CTAs on an SM: fewer, longer segments per CTA (a segment
+// of n rows loads n + 2) and independent step barriers, one CTA computing while another
+// waits, against the most march warps one CTA can have.  The choice is by a fit to the rates
+// measured with 2 to 14 segments and 1 to 6 CTAs per SM: an SM's rate grows by 20 units per
+// march warp and 55 per further CTA from 360.  It takes the fastest of k = 1 .. 6 on every
+// grid tried (Gcell-upd/s, k = 1 first): 61x31 257 -> 620 (k = 6), 81x41 382 -> 658 (3), 101x76
+// in clusters of two 328 -> 570 (3), 201x101 in clusters of three 446 -> 540 (2); one CTA on
+// 121x61 (542), 151x76 (636) and everything larger.
+static ResShape resident_shape(const Geometry &g, int C, int kmax = 1)
 {
     ResShape r{};
     const int npair = (g.nx + 1) / 2;
@@ -396,8 +419,20 @@ static ResShape resident_shape(const Geometry &g, int C)
     const size_t smem = (size_t)2 * R * sq * sizeof(float4) + (size_t)R * sizeof(KP) +
                         2 * kPatch * kPatch * sizeof(float);
     if (smem > 227 * 1024) return r;
-    int nseg = (kResThreads - 32) / npair;   // the last warp is the edge warp
-    if (nseg > R) nseg = R;
+    int nseg = 1;
+    double best = 0.0;
+    for (int k = 1; k <= kmax && k <= 10 && k * (smem + 1024) <= kSmemPerSm; k++) {
+        const int warps = kResThreads / 32 / k;   // of one CTA; the last one is the edge warp
+        const int most = (warps - 1) * 32 / npair;
+        if (most < 1) break;
+        const int rows = (R + (most < R ? most : R) - 1) / (most < R ? most : R);
+        const int n = (R + rows - 1) / rows;      // segments that have rows
+        const double score = (360.0 + 20.0 * k * ((npair * n + 31) / 32) + 55.0 * (k - 1)) * rows / (rows + 2.0);
+        if (score > best) {
+            best = score;
+            nseg = n;
+        }
+    }
     r.C = C;
     r.R = R;
     r.sq = sq;
@@ -424,6 +459,10 @@ int resident_cluster_size(const oed_ctx *ctx)
     return ctx->precision == OED_FP32 ? resident_fits(ctx->g) : 0;
 }
 
+using ResKernel = void (*)(ResArgs);
+static const ResKernel kResKernels[4] = {k_resident<false, false>, k_resident<false, true>, k_resident<true, false>,
+                                         k_resident<true, true>};
+
 // The kernel's dynamic shared-memory limit is always set to the device's opt-in
 // maximum (launches may use less): a fixed value, so concurrent callers with
 // different grids never lower it under each other.
@@ -432,7 +471,19 @@ static cudaError_t set_smem_limit()
     int dev = 0, optin = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    return cudaFuncSetAttribute(k_resident, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
+    for (ResKernel k : kResKernels) {
+        const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+static ResKernel resident_kernel(const oed_ctx *ctx, int C)
+{
+    bool hom = true;
+    for (size_t l = 1; l < ctx->vp.size(); l++)
+        hom &= ctx->vp[l] == ctx->vp[0] && ctx->vs[l] == ctx->vs[0] && ctx->rho[l] == ctx->rho[0];
+    return kResKernels[2 * hom + (C == 1)];
 }
 
 int resident_max_active_clusters(const oed_ctx *ctx, int C)
@@ -452,7 +503,7 @@ int resident_max_active_clusters(const oed_ctx *ctx, int C)
     cfg.attrs = at;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, k_resident, &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&n, resident_kernel(ctx, C), &cfg) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
@@ -463,7 +514,10 @@ int resident_max_active_clusters(const oed_ctx *ctx, int C)
 cudaError_t launch_resident(const oed_ctx *ctx, int C, int nsolve, cudaStream_t st, cudaEvent_t ev0,
                             cudaEvent_t ev1, int nsteps_override)
 {
-    const ResShape r = resident_shape(ctx->g, C);
+    int dev = 0, nsm = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    const ResShape r = resident_shape(ctx->g, C, (int)(((long long)nsolve * C + nsm - 1) / nsm));
     if (!r.C) return cudaErrorInvalidValue;
     set_smem_limit();
     ResArgs a;
@@ -493,7 +547,7 @@ cudaError_t launch_resident(const oed_ctx *ctx, int C, int nsolve, cudaStream_t 
     cfg.attrs = at;
     cfg.numAttrs = 1;
     if (ev0) cudaEventRecord(ev0, st);
-    cudaError_t e = cudaLaunchKernelEx(&cfg, k_resident, a);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, resident_kernel(ctx, C), a);
     if (ev1) cudaEventRecord(ev1, st);
     return e;
 }
