@@ -21,6 +21,8 @@
 //
 // The same launch gathers the receiver samples of level m from its input u^m
 // (Eq. forward_model), so the seismograms need no extra pass over the field.
+#include <algorithm>
+
 #include "stencil_cell.cuh"
 
 namespace oed {
@@ -117,6 +119,141 @@ __global__ void __launch_bounds__(256) k_step(StepArgs<real> a)
     }
 }
 
+// The FP64 step.  FP64 runs at two lanes per clock and SM here, 64 times below FP32, so a
+// warp's FP64 instruction holds its scheduler's pipe for 64 clocks: the pipe bounds the
+// kernel and everything else (loads, selects, index arithmetic) is free beside it.  The
+// split therefore saves FP64 issue slots only:
+//  - a thread owns a column pair (the first difference between its columns serves both) and
+//    up to ZS rows, each row's differences formed once as it enters as the south row;
+//  - threads are packed densely over (solve, row segment, pair), so no lanes idle at the right
+//    edge of a grid, and the segments of a grid are equally long to one row;
+//  - the surface row, the bottom row and the side columns take the slots of the interior
+//    update with selected operands instead of branches of their own (the rounding is that of
+//    node_update in each case).
+// 81x41, 240 solves: 25 slots per cell-update against 38 for the kernel of one column and
+// four rows per thread that it replaces.
+struct Row64 {
+    double ca[2], cb[2];   // centre values, u_x then u_z
+    double da[2], db[2];   // east - west differences
+    double va[2], vb[2];   // south row minus this row
+};
+
+template <int ZS>
+__global__ void __launch_bounds__(256) k_step64(StepArgs<double> a, int npair, int nseg, unsigned nthr)
+{
+    const Geometry &g = a.g;
+    const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
+    const int nq = 2 * g.nrec;
+    const unsigned per = (unsigned)npair * (unsigned)nseg;
+    if (t >= nthr) return;
+    const int s = (int)(t / per);
+    const unsigned w = t - (unsigned)s * per;
+    const int seg = (int)(w / (unsigned)npair), p = (int)(w - (unsigned)seg * (unsigned)npair);
+    const size_t base = (size_t)s * g.solve_stride;
+    const double *__restrict__ cur = a.cur + base;
+    double *__restrict__ nxt = a.nxt + base;
+    if (seg == 0)   // receiver samples of level m (the input field)
+        for (int q = p; q < nq; q += npair)
+            a.trace[((size_t)s * g.nlev + a.m) * nq + q] = cur[(q & 1) * g.comp_stride + a.rec[q >> 1]];
+
+    const int c = 2 * p, last = g.nx - 1;
+    const int j0 = (int)((long long)g.nz * seg / nseg), j1 = (int)((long long)g.nz * (seg + 1) / nseg);
+    const bool sideA = c == 0 || c == last, sideB = c + 1 == last, hasB = c + 1 <= last;
+    const int iw = c > 0 ? c - 1 : 0, ie = c + 2 <= last ? c + 2 : last;
+    // row j of u^m as seen by the pair; outside the grid the neighbour is the node itself
+    auto load = [&](int j, Row64 &r, double (&la)[2], double (&lb)[2]) {
+        const size_t o = (size_t)(j < g.nz - 1 ? j : g.nz - 1) * g.xp;
+#pragma unroll
+        for (int k = 0; k < 2; k++) {
+            const double *u = cur + k * g.comp_stride + o;
+            const double2 v = __ldg(reinterpret_cast<const double2 *>(u + c));
+            const double xw = __ldg(u + iw), xe = __ldg(u + ie);
+            const double xb = hasB ? v.y : v.x;
+            r.ca[k] = v.x;
+            r.cb[k] = xb;
+            const double f = xb - v.x;
+            la[k] = f - (v.x - xw);
+            lb[k] = (xe - xb) - f;
+            r.da[k] = xb - xw;
+            r.db[k] = xe - v.x;
+        }
+    };
+    auto south = [](Row64 &n, const Row64 &s_) {
+#pragma unroll
+        for (int k = 0; k < 2; k++) {
+            n.va[k] = s_.ca[k] - n.ca[k];
+            n.vb[k] = s_.cb[k] - n.cb[k];
+        }
+    };
+    // u^{m+1} of one component at one node: K1 .. K5 the operator's coefficients in op_x's order
+    auto node = [](double K1, double K2, double K3, double K4, double K5, double cside, double cbot, double uc, double um,
+                   double lap, double vs, double vn, double ds, double dn, bool side, bool bottom) {
+        const double a1 = fma(side ? cside : K1, lap, side ? uc : uc - um);
+        const double a2 = fma(K2, vs, a1);
+        const double a3 = fma(bottom ? -cbot : K3, vn, bottom ? uc : a2);
+        const double a5 = fma(K5, dn, fma(K4, ds, a3));
+        const double u = uc + a5;
+        return side ? a1 : (bottom ? a3 : u);
+    };
+    const int sj = a.src[s].j0, si = c - a.src[s].i0;
+    const bool scolA = (unsigned)si < (unsigned)kPatch, scolB = hasB && (unsigned)(si + 1) < (unsigned)kPatch;
+    const double S = scolA || scolB ? a.stf[(size_t)s * g.nsteps + a.m] : 0.0;
+
+    Row64 n, ce, so;
+    double la[2], lb[2], sa[2], sb[2];
+    load(j0, ce, la, lb);
+    if (j0 == 0) {   // no north differences, cross terms on the row itself
+        n = ce;
+#pragma unroll
+        for (int k = 0; k < 2; k++) n.va[k] = n.vb[k] = 0.0;
+    } else {
+        load(j0 - 1, n, sa, sb);
+        south(n, ce);
+    }
+#pragma unroll
+    for (int i = 0; i < ZS; i++) {
+        const int j = j0 + i;
+        if (j >= j1) break;
+        const bool bottom = j == g.nz - 1;
+        const FacCoef<double> K = a.fac[j];
+        const size_t o = (size_t)j * g.xp + c;
+        const double2 mx = __ldcs(reinterpret_cast<const double2 *>(nxt + o));
+        const double2 mz = __ldcs(reinterpret_cast<const double2 *>(nxt + g.comp_stride + o));
+        load(j + 1, so, sa, sb);
+        south(ce, so);
+        double xa = node(K.axx, K.axzp, K.naxzm, K.px, K.nqx, K.cp, K.cs, ce.ca[0], mx.x, la[0], ce.va[0], n.va[0],
+                         so.da[1], n.da[1], sideA, bottom);
+        double za = node(K.azx, K.azzp, K.nazzm, K.pz, K.nqz, K.cs, K.cp, ce.ca[1], mz.x, la[1], ce.va[1], n.va[1],
+                         so.da[0], n.da[0], sideA, bottom);
+        double xb = node(K.axx, K.axzp, K.naxzm, K.px, K.nqx, K.cp, K.cs, ce.cb[0], mx.y, lb[0], ce.vb[0], n.vb[0],
+                         so.db[1], n.db[1], sideB, bottom);
+        double zb = node(K.azx, K.azzp, K.nazzm, K.pz, K.nqz, K.cs, K.cp, ce.cb[1], mz.y, lb[1], ce.vb[1], n.vb[1],
+                         so.db[0], n.db[0], sideB, bottom);
+        const int b = j - sj;
+        if ((unsigned)b < (unsigned)kPatch && (scolA || scolB)) {
+            const SourceDesc<double> &d = a.src[s];
+            if (scolA) {
+                xa = add_force(xa, S, d.wx[b * kPatch + si]);
+                za = add_force(za, S, d.wz[b * kPatch + si]);
+            }
+            if (scolB) {
+                xb = add_force(xb, S, d.wx[b * kPatch + si + 1]);
+                zb = add_force(zb, S, d.wz[b * kPatch + si + 1]);
+            }
+        }
+        if (!hasB) xb = zb = 0.0;   // the padding column stays zero
+        __stcs(reinterpret_cast<double2 *>(nxt + o), make_double2(xa, xb));
+        __stcs(reinterpret_cast<double2 *>(nxt + g.comp_stride + o), make_double2(za, zb));
+        n = ce;
+        ce = so;
+#pragma unroll
+        for (int k = 0; k < 2; k++) {
+            la[k] = sa[k];
+            lb[k] = sb[k];
+        }
+    }
+}
+
 // Receiver samples of one level (used for the last level after the final step).
 template <typename real>
 __global__ void k_gather(const real *__restrict__ cur, real *__restrict__ trace,
@@ -131,15 +268,40 @@ __global__ void k_gather(const real *__restrict__ cur, real *__restrict__ trace,
         tr[q] = (q & 1 ? cz : cx)[rec[q >> 1]];
 }
 
+// One step of nsolve solves with the context's launch shape.
+template <typename real, int ZS>
+static void launch_one(const oed_ctx *ctx, int nsolve, const StepArgs<real> &a, cudaStream_t st)
+{
+    const Geometry &g = ctx->g;
+    const int wz = ctx->tune.wz;
+    if constexpr (sizeof(real) == 8) {
+        const int npair = (g.nx + 1) / 2, nseg = (g.nz + ZS - 1) / ZS;
+        const long long per = (long long)npair * nseg;
+        // 32-bit thread numbers: a batch past them goes in several launches
+        const int most = (int)std::max(1LL, std::min((long long)nsolve, (1LL << 31) / per));
+        for (int s0 = 0; s0 < nsolve; s0 += most) {
+            const int ns = std::min(most, nsolve - s0);
+            StepArgs<double> b = a;
+            b.cur += (size_t)s0 * g.solve_stride;
+            b.nxt += (size_t)s0 * g.solve_stride;
+            b.src += s0;
+            b.stf += (size_t)s0 * g.nsteps;
+            b.trace += (size_t)s0 * g.nlev * g.nrec * 2;
+            const unsigned nthr = (unsigned)(per * ns);
+            k_step64<ZS><<<(nthr + 32 * wz - 1) / (32 * wz), 32 * wz, 0, st>>>(b, npair, nseg, nthr);
+        }
+    } else {
+        const int rows_per_block = wz * ZS;
+        dim3 grid((g.nx + 31) / 32, (g.nz + rows_per_block - 1) / rows_per_block, nsolve);
+        k_step<real, ZS><<<grid, dim3(32, wz), 0, st>>>(a);
+    }
+}
+
 template <typename real, int ZS>
 static void launch_steps_zs(const oed_ctx *ctx, int nsolve, cudaStream_t st, cudaEvent_t ev0,
                             cudaEvent_t ev1)
 {
     const Geometry &g = ctx->g;
-    const int wz = ctx->tune.wz;
-    dim3 block(32, wz);
-    const int rows_per_block = wz * ZS;
-    dim3 grid((g.nx + 31) / 32, (g.nz + rows_per_block - 1) / rows_per_block, nsolve);
     real *u0 = (real *)ctx->d_u0, *u1 = (real *)ctx->d_u1;
     StepArgs<real> a;
     a.fac = (const FacCoef<real> *)ctx->d_fac;
@@ -154,7 +316,7 @@ static void launch_steps_zs(const oed_ctx *ctx, int nsolve, cudaStream_t st, cud
         a.cur = (m & 1) ? u1 : u0;
         a.nxt = (m & 1) ? u0 : u1;
         a.m = m;
-        k_step<real, ZS><<<grid, block, 0, st>>>(a);
+        launch_one<real, ZS>(ctx, nsolve, a, st);
     }
     if (ev1) cudaEventRecordWithFlags(ev1, st, cudaEventRecordExternal);
     const real *last = (g.nsteps & 1) ? u1 : u0;
@@ -180,10 +342,6 @@ static void probe_zs(const oed_ctx *ctx, int nsolve, int nrep, cudaStream_t st, 
                      cudaEvent_t ev1)
 {
     const Geometry &g = ctx->g;
-    const int wz = ctx->tune.wz;
-    dim3 block(32, wz);
-    const int rows_per_block = wz * ZS;
-    dim3 grid((g.nx + 31) / 32, (g.nz + rows_per_block - 1) / rows_per_block, nsolve);
     StepArgs<real> a;
     a.fac = (const FacCoef<real> *)ctx->d_fac;
     a.src = (const SourceDesc<real> *)ctx->d_src;
@@ -196,7 +354,7 @@ static void probe_zs(const oed_ctx *ctx, int nsolve, int nrep, cudaStream_t st, 
         a.cur = (real *)((m & 1) ? ctx->d_u1 : ctx->d_u0);
         a.nxt = (real *)((m & 1) ? ctx->d_u0 : ctx->d_u1);
         a.m = m % g.nsteps;
-        k_step<real, ZS><<<grid, block, 0, st>>>(a);
+        launch_one<real, ZS>(ctx, nsolve, a, st);
     }
     cudaEventRecord(ev1, st);
 }
