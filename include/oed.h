@@ -307,8 +307,11 @@ int oed_hessian_map(oed_ctx *ctx, double *theta, int n, const double *y, const d
  * (Sec. 4.4 compares the two).  With y_n = g_outer[n] + eps[n] and noise sigma^2 I,
  *   log_ev[n] = log( (1/M) sum_m exp(-|y_n - g_inner[m]|^2 / (2 sigma^2)) )
  *   eig       = (1/N) sum_n ( -|eps_n|^2 / (2 sigma^2) - log_ev[n] )
- * (the Gaussian normalising constant cancels).  FP64 throughout; distances are
- * summed from the differences (no |y|^2 + |g|^2 - 2 y.g expansion).
+ * (the Gaussian normalising constant cancels).  Distances are summed in FP64 from
+ * the differences (no |y|^2 + |g|^2 - 2 y.g expansion); inner samples whose terms a
+ * rigorous FP32 bound puts below 2^-60 of a row's sum, all of them together, are left
+ * out.  Scratch is allocated stream-ordered for the call (2^25 floats of distances at
+ * most, and the data in FP32); where it does not fit every pair is summed.
  *   g_outer  device [N][D]  noise-free data of the outer samples, e.g. seismograms
  *                           from oed_forward (D = (nsteps+1) * nrec * 2)
  *   eps      device [N][D]  the noise realisations (the caller draws them)

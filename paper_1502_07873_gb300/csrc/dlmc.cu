@@ -8,109 +8,282 @@
 // squared distances summed from the differences themselves (no |y|^2 + |g|^2 - 2 y.g
 // expansion, which cancels catastrophically when the noise is small).
 //
-// k_log_evidence: a block owns 32 outer samples and streams all inner samples in
-// tiles of 64, the data dimension in chunks of 32 through shared memory; each
-// thread accumulates a 2 x 4 tile of squared distances, then folds them into a
-// running (max, sum of exponentials) per outer sample; the 16 threads sharing an
-// outer sample combine their partial sums with shuffles at the end.
+// FP64 runs 64 times slower than FP32 here, and only the inner samples near a row's best
+// contribute to its log-sum-exp: k_screen computes every distance in FP32 (of values scaled
+// by 1 / (sigma sqrt 2), so a distance is -l), and k_log_evidence computes in FP64 those that
+// can matter.  A pair (n, m) is left out only when a rigorous lower bound of its distance,
+// from its FP32 value, exceeds an upper bound of the row's smallest by
+// (kDropBits + log2 M) ln 2: all left-out terms together are then below 2^-kDropBits of the
+// sum's largest term, far below the rounding of the sum.  With u = 2^-24, rounding the scaled
+// inputs moves a distance's root by at most eta = u (|y_n| + max_m |g_m|) (and 1e-22 where
+// they underflow), the FP32 sum of squares its value by a factor within 1 +- (D + 8) u.
+// Values that FP32 cannot hold (overflow, NaN) are always kept.
+//
+// Both sides measured (N = M = 4096, sigma = 0.01, the paper's study): D = 204, where 1.3% of the
+// pairs are kept, 17.8 ms with every pair in FP64 (two FP64 operations a pair and entry, tiles of
+// 32 x 64) and 0.91 ms screened (0.33 the FP32 distances, about 0.45 the FP64 part); D = 72,
+// records that end before the waves arrive and every pair matters, 8.0 and 5.3 ms.
 #include <math.h>
+
+#include <algorithm>
+#include <cmath>
 
 #include "oed_internal.cuh"
 
 namespace oed {
 
-constexpr int kDN = 32, kDM = 64, kDD = 32;
+constexpr int kSN = 64, kSM = 64, kSD = 32;      // k_screen: block tile and chunk of the data dimension
+constexpr int kDropBits = 60;
+constexpr size_t kScreenFloats = (size_t)1 << 25;   // distances held at once (128 MB); rows go in groups
 
-__global__ void __launch_bounds__(256) k_log_evidence(const double *__restrict__ g_out,
-                                                      const double *__restrict__ eps, int N,
-                                                      const double *__restrict__ g_in, int M, int D,
-                                                      double inv2s2, double *__restrict__ log_ev)
+// y_n = g_outer[n] + eps[n], scaled and rounded to FP32; g likewise
+__device__ __forceinline__ float screen_value(double v, double scale) { return (float)(v * scale); }
+
+// The screened values, rows padded with zeros to Dp entries: y of the rows below N, -g of the
+// next M rows (a sum is then the difference), and max_m |g_m| as the bits of a float (rounded
+// up).  One warp per row.
+__global__ void __launch_bounds__(256) k_screen_values(const double *__restrict__ g_out, const double *__restrict__ eps,
+                                                       int N, const double *__restrict__ g_in, int M, int D, int Dp,
+                                                       double scale, float *__restrict__ val, unsigned *__restrict__ gmax)
 {
-    __shared__ double ys[kDD][kDN];
-    __shared__ double gs[kDD][kDM + 1];
-    const int tid = threadIdx.x;
-    const int tx = tid % 16, ty = tid / 16;
-    const int n0 = blockIdx.x * kDN;
-    double mx[2] = {-INFINITY, -INFINITY}, sm[2] = {0.0, 0.0};
-    for (int m0 = 0; m0 < M; m0 += kDM) {
-        double acc[2][4];
-#pragma unroll
-        for (int r = 0; r < 2; r++)
-#pragma unroll
-            for (int q = 0; q < 4; q++) acc[r][q] = 0.0;
-        for (int d0 = 0; d0 < D; d0 += kDD) {
-            // y tile (32 x 32): y = g(theta_n) + eps_n, zero outside the data
-            for (int k = tid; k < kDN * kDD; k += 256) {
-                const int nn = k / kDD, dd = k % kDD;
-                const int n = n0 + nn, d = d0 + dd;
-                double v = 0.0;
-                if (n < N && d < D) v = g_out[(size_t)n * D + d] + eps[(size_t)n * D + d];
-                ys[dd][nn] = v;
-            }
-            for (int k = tid; k < kDM * kDD; k += 256) {
-                const int mm = k / kDD, dd = k % kDD;
-                const int m = m0 + mm, d = d0 + dd;
-                gs[dd][mm] = (m < M && d < D) ? g_in[(size_t)m * D + d] : 0.0;
-            }
-            __syncthreads();
-#pragma unroll 4
-            for (int dd = 0; dd < kDD; dd++) {
-                const double a0 = ys[dd][2 * ty], a1 = ys[dd][2 * ty + 1];
-#pragma unroll
-                for (int q = 0; q < 4; q++) {
-                    const double b = gs[dd][tx + 16 * q];
-                    const double e0 = a0 - b, e1 = a1 - b;
-                    acc[0][q] = fma(e0, e0, acc[0][q]);
-                    acc[1][q] = fma(e1, e1, acc[1][q]);
-                }
-            }
-            __syncthreads();
-        }
-#pragma unroll
-        for (int q = 0; q < 4; q++) {
-            if (m0 + tx + 16 * q >= M) continue;
-#pragma unroll
-            for (int r = 0; r < 2; r++) {
-                const double l = -acc[r][q] * inv2s2;
-                if (l > mx[r]) {
-                    sm[r] = sm[r] * exp(mx[r] - l) + 1.0;
-                    mx[r] = l;
-                } else {
-                    sm[r] += exp(l - mx[r]);
-                }
-            }
-        }
+    const int r = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (r >= N + M) return;
+    float s = 0.0f;
+    for (int d = lane; d < Dp; d += 32) {
+        float v = 0.0f;
+        if (d < D) v = r < N ? screen_value(g_out[(size_t)r * D + d] + eps[(size_t)r * D + d], scale)
+                             : -screen_value(g_in[(size_t)(r - N) * D + d], scale);
+        val[(size_t)r * Dp + d] = v;
+        s = fmaf(v, v, s);
     }
-    // combine the 16 threads of each outer sample (lanes differing in the low four bits)
+    if (r < N) return;
 #pragma unroll
-    for (int r = 0; r < 2; r++) {
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    // the sum's rounding is within (D + 8) u as above; NaN and overflow raise the bound to infinity
+    const float q = sqrtf(s) * (1.0f + (D + 8) * 6e-8f);
+    if (lane == 0) atomicMax(gmax, __float_as_uint(q <= 3e38f ? q : INFINITY));
+}
+
+// dist[n - n0][m] = |y_n - g_m|^2 in FP32 for the rows n0 .. n1 - 1, and per row the bits of the
+// smallest (finite) one.  A thread owns a 4 x 4 tile and two data entries at a time (.f32x2).
+__global__ void __launch_bounds__(256) k_screen(const float *__restrict__ val, int N, int n0, int n1, int M, int Dp,
+                                                float *__restrict__ dist, unsigned *__restrict__ best)
+{
+    __shared__ float2 ys[kSD / 2][kSN + 1], gs[kSD / 2][kSM + 1];
+    const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
+    const int nb = n0 + blockIdx.y * kSN, mb = blockIdx.x * kSM;
+    const float *gval = val + (size_t)N * Dp;
+    float2 acc[4][4];
 #pragma unroll
-        for (int off = 8; off > 0; off >>= 1) {
-            const double om = __shfl_xor_sync(0xffffffffu, mx[r], off);
-            const double os = __shfl_xor_sync(0xffffffffu, sm[r], off);
-            const double nm = fmax(mx[r], om);
-            double ns = 0.0;
-            if (nm > -INFINITY) ns = sm[r] * exp(mx[r] - nm) + os * exp(om - nm);
-            mx[r] = nm;
-            sm[r] = ns;
+    for (int i = 0; i < 4; i++)
+#pragma unroll
+        for (int j = 0; j < 4; j++) acc[i][j] = make_float2(0.0f, 0.0f);
+    for (int d0 = 0; d0 < Dp; d0 += kSD) {
+#pragma unroll
+        for (int q = 0; q < kSN * kSD / 256; q++) {
+            const int k = tid + 256 * q, r = k / kSD, c = k % kSD;
+            const float y = nb + r < n1 ? val[(size_t)(nb + r) * Dp + d0 + c] : 0.0f;
+            const float g = mb + r < M ? gval[(size_t)(mb + r) * Dp + d0 + c] : 0.0f;
+            (&ys[c >> 1][r].x)[c & 1] = y;
+            (&gs[c >> 1][r].x)[c & 1] = g;
         }
-        const int n = n0 + 2 * ty + r;
-        if (tx == 0 && n < N) log_ev[n] = mx[r] + log(sm[r]) - log((double)M);
+        __syncthreads();
+#pragma unroll 4
+        for (int c = 0; c < kSD / 2; c++) {
+            float2 y[4], g[4];
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+                y[i] = ys[c][ty + 16 * i];
+                g[i] = gs[c][tx + 16 * i];
+            }
+#pragma unroll
+            for (int i = 0; i < 4; i++)
+#pragma unroll
+                for (int j = 0; j < 4; j++) {
+                    const float2 e = __fadd2_rn(y[i], g[j]);
+                    acc[i][j] = __ffma2_rn(e, e, acc[i][j]);
+                }
+        }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+        const int n = nb + ty + 16 * i;
+        float b = INFINITY;
+        if (n < n1)
+#pragma unroll
+            for (int j = 0; j < 4; j++) {
+                const int m = mb + tx + 16 * j;
+                if (m >= M) continue;
+                const float v = acc[i][j].x + acc[i][j].y;
+                dist[(size_t)(n - n0) * M + m] = v;
+                b = fminf(b, v);   // ignores NaN
+            }
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) b = fminf(b, __shfl_xor_sync(0xffffffffu, b, o));
+        if (tx == 0 && n < n1) atomicMin(best + n, __float_as_uint(b));
     }
 }
 
-// I_DL = (1/N) sum_n [-|eps_n|^2 inv2s2 - log_ev[n]]: one block, fixed summation order.
-__global__ void __launch_bounds__(512) k_dlmc_sum(const double *__restrict__ eps, const double *__restrict__ log_ev,
-                                                  int N, int D, double inv2s2, double *__restrict__ eig)
+// log_ev[n], one block per row: collect the samples to keep, 32 at a time and a lane each, sum
+// their squared differences in FP64 in the order of the data, and fold them into a running
+// (max, sum of exponentials) per lane; e2[n] = |eps_n|^2 where asked for.  dist NULL: all are kept.
+constexpr int kEvWarps = 4, kEvPer = 8, kEvList = 2048;   // warps, samples a lane looks at per round, list
+constexpr int kEvShared = 12288;   // longest data row kept in shared memory (96 KB)
+
+// (max, sum) of a warp's lanes; every lane gets them
+__device__ __forceinline__ void warp_log_sum(double &mx, double &sm)
+{
+    double top = mx;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) top = fmax(top, __shfl_xor_sync(0xffffffffu, top, o));
+    double s = top > -INFINITY ? sm * exp(mx - top) : 0.0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    mx = top;
+    sm = s;
+}
+
+template <bool SHARED>
+__global__ void __launch_bounds__(32 * kEvWarps) k_log_evidence(
+    const double *__restrict__ g_out, const double *__restrict__ eps, int n0, const double *__restrict__ g_in, int M, int D,
+    int Dp, double inv2s2, double log_m, float slack, const float *__restrict__ val, const float *__restrict__ dist,
+    const unsigned *__restrict__ best, const unsigned *__restrict__ gmax, int vec, double *__restrict__ log_ev,
+    double *__restrict__ e2)
+{
+    extern __shared__ double ys[];   // [D] this row's data
+    __shared__ int list[kEvList];
+    __shared__ int wcount[kEvWarps];
+    __shared__ double red[2][kEvWarps];
+    __shared__ float rednorm[kEvWarps];
+    const int n = n0 + blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    float ynorm = 0.0f;
+    double e = 0.0;
+    for (int d = tid; d < D; d += blockDim.x) {
+        const double ep = eps[(size_t)n * D + d];
+        if (SHARED) ys[d] = g_out[(size_t)n * D + d] + ep;
+        e = fma(ep, ep, e);
+        if (dist) {
+            const float v = val[(size_t)n * Dp + d];
+            ynorm = fmaf(v, v, ynorm);
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        ynorm += __shfl_xor_sync(0xffffffffu, ynorm, o);
+        e += __shfl_xor_sync(0xffffffffu, e, o);
+    }
+    if (lane == 0) {
+        red[0][warp] = e;
+        rednorm[warp] = ynorm;
+    }
+    __syncthreads();
+    float limit = INFINITY;   // keep distances up to this
+    if (dist) {
+        float y2 = 0.0f;
+        for (int k = 0; k < kEvWarps; k++) y2 += rednorm[k];
+        if (e2 && tid == 0) e2[n] = (red[0][0] + red[0][1]) + (red[0][2] + red[0][3]);
+        // every operation rounds the limit up
+        const float u = 5.9604644775390625e-08f, kappa = (D + 8) * u, up = __fadd_ru(1.0f, __fmul_ru(kappa, 1.001f));
+        const float eta = __fadd_ru(__fmul_ru(__fmul_ru(u, 1.001f), __fadd_ru(__fmul_ru(__fsqrt_ru(y2), up),
+                                                                             __uint_as_float(*gmax))), 1e-22f * D);
+        const float lo = __fadd_ru(__fmul_ru(__fsqrt_ru(__uint_as_float(best[n])), up), eta);
+        const float root = __fdiv_ru(__fadd_ru(__fsqrt_ru(__fadd_ru(__fmul_ru(lo, lo), slack)), eta),
+                                     __fadd_rd(1.0f, -1.001f * kappa));
+        const float lim = __fmul_ru(root, root);
+        if (lim < 1e38f && kappa < 0.01f) limit = lim;
+    }
+    auto data = [&](int d) { return SHARED ? ys[d] : g_out[(size_t)n * D + d] + eps[(size_t)n * D + d]; };
+    double mx = -INFINITY, sm = 0.0;
+    const float *row = dist ? dist + (size_t)blockIdx.x * M : nullptr;
+    for (int m0 = 0; m0 < M;) {
+        // the next samples to keep, in order, up to a full list
+        int have = 0;
+        __syncthreads();
+        while (m0 < M && have + kEvPer * (int)blockDim.x <= kEvList) {
+            // a warp takes kEvPer x 32 consecutive samples; kept unless known to be above the
+            // limit (NaN and overflow are kept)
+            unsigned b[kEvPer];
+            int mine = 0;
+#pragma unroll
+            for (int q = 0; q < kEvPer; q++) {
+                const int m = m0 + (warp * kEvPer + q) * 32 + lane;
+                const float v = row && m < M ? row[m] : 0.0f;
+                b[q] = __ballot_sync(0xffffffffu, m < M && (!(v > limit) || !(v < 3e38f)));
+                mine += __popc(b[q]);
+            }
+            if (lane == 0) wcount[warp] = mine;
+            __syncthreads();
+            int at = have;
+            for (int k = 0; k < kEvWarps; k++) {
+                if (k < warp) at += wcount[k];
+                have += wcount[k];
+            }
+#pragma unroll
+            for (int q = 0; q < kEvPer; q++) {
+                if (b[q] >> lane & 1) list[at + __popc(b[q] & ((1u << lane) - 1u))] = m0 + (warp * kEvPer + q) * 32 + lane;
+                at += __popc(b[q]);
+            }
+            m0 += kEvPer * (int)blockDim.x;
+            __syncthreads();
+        }
+        for (int k = tid; k < have; k += blockDim.x) {
+            const double *g = g_in + (size_t)list[k] * D;
+            double acc = 0.0;
+            int d = 0;
+            if (vec)
+#pragma unroll 4
+                for (; d < D; d += 2) {
+                    const double2 v = *reinterpret_cast<const double2 *>(g + d);
+                    const double a0 = data(d) - v.x, a1 = data(d + 1) - v.y;
+                    acc = fma(a0, a0, acc);
+                    acc = fma(a1, a1, acc);
+                }
+            for (; d < D; d++) {
+                const double a0 = data(d) - g[d];
+                acc = fma(a0, a0, acc);
+            }
+            const double l = -acc * inv2s2;
+            const double t = exp(-fabs(l - mx));
+            if (l > mx) {
+                sm = sm * t + 1.0;
+                mx = l;
+            } else if (!(l == -INFINITY)) {   // (an infinite distance adds nothing)
+                sm += t;
+            }
+        }
+    }
+    // combine the lanes, then the warps
+    if (__any_sync(0xffffffffu, mx > -INFINITY || sm != 0.0)) warp_log_sum(mx, sm);
+    if (lane == 0) {
+        red[0][warp] = mx;
+        red[1][warp] = sm;
+    }
+    __syncthreads();
+    if (warp == 0) {
+        mx = lane < kEvWarps ? red[0][lane] : -INFINITY;
+        sm = lane < kEvWarps ? red[1][lane] : 0.0;
+        warp_log_sum(mx, sm);
+        if (lane == 0) log_ev[n] = mx + log(sm) - log_m;
+    }
+}
+
+// I_DL = (1/N) sum_n [-|eps_n|^2 inv2s2 - log_ev[n]]: one block, fixed summation order; e2 NULL:
+// the squared norms of the noise are summed here
+__global__ void __launch_bounds__(512) k_dlmc_sum(const double *__restrict__ eps, const double *__restrict__ e2,
+                                                  const double *__restrict__ log_ev, int N, int D, double inv2s2,
+                                                  double *__restrict__ eig)
 {
     __shared__ double sv[512];
     const int t = threadIdx.x, T = blockDim.x;
-    const int per = (N + T - 1) / T;
     double v = 0.0;
-    for (int n = t * per; n < (t + 1) * per && n < N; n++) {
-        double e2 = 0.0;
-        for (int d = 0; d < D; d++) e2 = fma(eps[(size_t)n * D + d], eps[(size_t)n * D + d], e2);
-        v += -e2 * inv2s2 - log_ev[n];
+    for (int n = t; n < N; n += T) {
+        double q = 0.0;
+        if (e2)
+            q = e2[n];
+        else
+            for (int d = 0; d < D; d++) q = fma(eps[(size_t)n * D + d], eps[(size_t)n * D + d], q);
+        v += -q * inv2s2 - log_ev[n];
     }
     sv[t] = v;
     __syncthreads();
@@ -130,8 +303,45 @@ extern "C" int oed_dlmc(const double *g_outer, const double *eps, int N, const d
     if (N < 1 || M < 1 || D < 1 || !g_outer || !eps || !g_inner || !log_ev || !(sigma > 0.0))
         return OED_EINVAL;
     cudaStream_t st = (cudaStream_t)stream;
-    const double inv2s2 = 1.0 / (2.0 * sigma * sigma);
-    k_log_evidence<<<(N + kDN - 1) / kDN, 256, 0, st>>>(g_outer, eps, N, g_inner, M, D, inv2s2, log_ev);
-    if (eig) k_dlmc_sum<<<1, 512, 0, st>>>(eps, log_ev, N, D, inv2s2, eig);
+    const double inv2s2 = 1.0 / (2.0 * sigma * sigma), scale = sqrt(inv2s2);
+    // scratch: [N] |eps|^2, the screened values, the distances of a group of rows, [N] smallest
+    // distances, the largest norm.  Without it (the device is full) every pair is kept, at more time.
+    const int Dp = (D + kSD - 1) / kSD * kSD;
+    const size_t held = std::min((size_t)N * M, kScreenFloats);
+    const int rows = (int)std::min((size_t)N, std::max(held / M / kSN * kSN, (size_t)kSN));
+    const size_t nval = ((size_t)N + M) * Dp, ndist = (size_t)rows * M;
+    double *e2 = nullptr;
+    if (cudaMallocAsync((void **)&e2, (size_t)N * 8 + (nval + ndist + N + 1) * 4, st) != cudaSuccess) {
+        cudaGetLastError();
+        e2 = nullptr;
+    }
+    float *val = e2 ? (float *)(e2 + N) : nullptr, *dist = e2 ? val + nval : nullptr;
+    unsigned *best = e2 ? (unsigned *)(dist + ndist) : nullptr, *gmax = e2 ? best + N : nullptr;
+    if (e2) {
+        cudaMemsetAsync(best, 0x7f, (size_t)N * 4, st);
+        cudaMemsetAsync(gmax, 0, 4, st);
+        k_screen_values<<<(unsigned)(((size_t)N + M + 7) / 8), 256, 0, st>>>(g_outer, eps, N, g_inner, M, D, Dp, scale,
+                                                                             val, gmax);
+    }
+    const int vec = D % 2 == 0 && (uintptr_t)g_inner % 16 == 0;
+    const bool shared = D <= kEvShared;
+    const double log_m = std::log((double)M);
+    const float slack = (float)((kDropBits * 0.6931471805599453 + log_m) * 1.000001);
+    if (shared)
+        cudaFuncSetAttribute(k_log_evidence<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kEvShared * 8);
+    for (int n0 = 0; n0 < N; n0 += rows) {
+        const int n1 = std::min(N, n0 + rows);
+        if (dist)
+            k_screen<<<dim3((M + kSM - 1) / kSM, (n1 - n0 + kSN - 1) / kSN), 256, 0, st>>>(val, N, n0, n1, M, Dp, dist,
+                                                                                          best);
+        if (shared)
+            k_log_evidence<true><<<n1 - n0, 32 * kEvWarps, (size_t)D * 8, st>>>(
+                g_outer, eps, n0, g_inner, M, D, Dp, inv2s2, log_m, slack, val, dist, best, gmax, vec, log_ev, e2);
+        else
+            k_log_evidence<false><<<n1 - n0, 32 * kEvWarps, 0, st>>>(
+                g_outer, eps, n0, g_inner, M, D, Dp, inv2s2, log_m, slack, val, dist, best, gmax, vec, log_ev, e2);
+    }
+    if (eig) k_dlmc_sum<<<1, 512, 0, st>>>(eps, e2, log_ev, N, D, inv2s2, eig);
+    if (e2) cudaFreeAsync(e2, st);
     return cudaGetLastError() == cudaSuccess ? OED_OK : OED_ECUDA;
 }
