@@ -9,6 +9,8 @@
 //    All of it in FP64, stored in the stencil's precision.
 //  - k_rows: per-row stencil coefficients of the leap-frog update for a medium
 //    layered in depth (lambda = rho (vp^2 - 2 vs^2), mu = rho vs^2, Sec. 2.1).
+#include <algorithm>
+
 #include "oed_internal.cuh"
 
 namespace oed {
@@ -82,29 +84,6 @@ struct FdStep {
     double d[kNT];
 };
 
-// Spatial part of M grad(delta) for one parameter vector on its 6x6 support:
-// corner (kx - 2, kz - 2); f[b][a] at node (kx - 2 + a, kz - 2 + b).
-//   f_x = m_xx delta'(x) delta(z) + m_xz delta(x) delta'(z)
-//   f_z = m_xz delta'(x) delta(z) + m_zz delta(x) delta'(z)
-// Returns false if x_s / h or z_s / h is not a usable number.
-__device__ bool source_patch6(const double *th, double h, int *kx, int *kz, double *fx, double *fz)
-{
-    const double qx = th[0] / h, qz = th[1] / h;
-    const double flx = floor(qx), flz = floor(qz);
-    if (!(isfinite(qx) && isfinite(qz) && fabs(flx) < 1e9 && fabs(flz) < 1e9)) return false;
-    double dx[6], dpx[6], dz[6], dpz[6];
-    delta_weights(qx - flx, h, dx, dpx);
-    delta_weights(qz - flz, h, dz, dpz);
-    *kx = (int)flx;
-    *kz = (int)flz;
-    for (int b = 0; b < 6; b++)
-        for (int a = 0; a < 6; a++) {
-            fx[b * 6 + a] = th[4] * dpx[a] * dz[b] + th[5] * dx[a] * dpz[b];
-            fz[b * 6 + a] = th[5] * dpx[a] * dz[b] + th[6] * dx[a] * dpz[b];
-        }
-    return true;
-}
-
 // S(t) of the given kind: OED_STF_GAUSS (Sec. 4.1, w = omega_s) or OED_STF_RICKER
 // ((1 - 2a) e^{-a}, a = (pi w (t - ts))^2, w the peak frequency)
 __device__ __forceinline__ double stf_value(int kind, double t, double ts, double ws)
@@ -118,140 +97,174 @@ __device__ __forceinline__ double stf_value(int kind, double t, double ts, doubl
     return ws * 0.3989422804014327 * exp(-0.5 * ws * ws * u * u);   // w / sqrt(2 pi) e^{...}
 }
 
-// One thread block per solve.  per_node = 1: the node itself (forward map);
+// All solves of one node.  per_node = 1: the node itself (forward map);
 // per_node = 15: centre and theta +/- d_j e_j (pairs Jacobian); per_node = 7:
 // solve j carries the FP64 difference of the theta + d_j e_j and theta - d_j e_j
 // forcings (difference Jacobian; by linearity of the scheme in the forcing its
-// seismogram is exactly g(theta + d_j e_j) - g(theta - d_j e_j)).  For j = x_s, z_s
-// and the moments the spatial patch differs (the two 6x6 patches are subtracted
-// on their 7x7 union); for j = t_s, omega_s the time function differs.
+// seismogram is exactly g(theta + d_j e_j) - g(theta - d_j e_j)), or with sens the analytic
+// derivative of the forcing (Alg. 1 step 2).  Spatial part of a solve on its 6x6 support,
+// corner (kx - 2, kz - 2), entry (b, a) at node (kx - 2 + a, kz - 2 + b):
+//   f_x = m_xx delta'(x) delta(z) + m_xz delta(x) delta'(z)
+//   f_z = m_xz delta'(x) delta(z) + m_zz delta(x) delta'(z)
+// For j = x_s, z_s and the moments the two 6x6 patches of a difference solve are subtracted
+// on their 7x7 union; for j = t_s, omega_s the time function differs.
+//
+// A node's solves share almost everything: at most three positions per axis (the node's and
+// the two perturbed ones, a lane each for the weights) and five time functions.  One block
+// per solve with one thread for its patch, and an exponential per solve and step, took
+// 0.80 ms for 2048 nodes of 7 solves of 50 steps (the FP64 pipe, mostly one lane of it);
+// this form 0.09 ms.  Block y of a node takes a part of its time steps, block 0 the patches too.
 template <typename real>
-__global__ void k_sources(const double *__restrict__ theta_nodes, int nsolve, int per_node, int sens,
-                          int stf_kind, FdStep step, Geometry g, const RowCoef<real> *__restrict__ rows,
-                          SourceDesc<real> *__restrict__ src, real *__restrict__ stf,
-                          double *__restrict__ theta_out)
+__global__ void __launch_bounds__(128) k_sources(const double *__restrict__ theta_nodes, int per_node, int sens,
+                                                 int stf_kind, FdStep step, Geometry g,
+                                                 const RowCoef<real> *__restrict__ rows,
+                                                 SourceDesc<real> *__restrict__ src, real *__restrict__ stf,
+                                                 double *__restrict__ theta_out)
 {
-    const int s = blockIdx.x;
-    if (s >= nsolve) return;
-    const int node = s / per_node, p = s % per_node;
-    const bool diff = per_node == kND && !sens;
-    __shared__ double th[kNT], tp[kNT], tm[kNT];
-    __shared__ double w7x[kPatch * kPatch], w7z[kPatch * kPatch];
-    __shared__ int corner[3];
-    __shared__ int time_diff;
-    __shared__ int time_kind;   // sensitivity solves: 0 S, 1 dS/dt_s, 2 dS/domega_s
-    if (threadIdx.x < kNT) {
-        const int j = threadIdx.x;
-        const double v = theta_nodes[(size_t)node * kNT + j];
-        double vs = v;
-        // pairs form: p = 0 centre, p = 1 + 2j: +d_j, p = 2 + 2j: -d_j
-        if (per_node == kNP && p > 0 && j == (p - 1) / 2) vs += ((p - 1) & 1) ? -step.d[j] : step.d[j];
-        th[j] = vs;
-        tp[j] = v + ((diff && j == p) ? step.d[j] : 0.0);
-        tm[j] = v - ((diff && j == p) ? step.d[j] : 0.0);
-        theta_out[(size_t)s * kNT + j] = vs;
+    const int node = blockIdx.x, tid = threadIdx.x;
+    const bool diff = per_node == kND && !sens, pairs = per_node == kNP;
+    __shared__ double th[kNT], thp[kNT], thm[kNT];   // the node, + d_j and - d_j in each entry
+    __shared__ double W[2][3][4][6];                 // axis, position (node, +, -), delta, delta', and their d/dx_s
+    __shared__ int cell[2][3], fin[2][3];            // first node of the weights + 2; usable position
+    __shared__ int corner[kNP][3];                   // patch corner and whether it fits, per solve
+    if (tid < kNT) {
+        const double v = theta_nodes[(size_t)node * kNT + tid];
+        th[tid] = v;
+        thp[tid] = v + step.d[tid];
+        thm[tid] = v - step.d[tid];
     }
-    for (int k = threadIdx.x; k < kPatch * kPatch; k += blockDim.x) w7x[k] = w7z[k] = 0.0;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double fx[36], fz[36];
-        int kx = 0, kz = 0, ok;
-        int i0, j0, span;   // span: 6 or 7 nodes of the patch actually used
-        time_diff = diff && (p == 2 || p == 3);
-        time_kind = (sens && (p == 2 || p == 3)) ? p - 1 : 0;
-        if (sens) {
-            // Alg. 1 step 2: the forcing of solve j is df/dtheta_j of the discrete source
-            const double qx = th[0] / g.h, qz = th[1] / g.h;
-            const double flx = floor(qx), flz = floor(qz);
-            ok = isfinite(qx) && isfinite(qz) && fabs(flx) < 1e9 && fabs(flz) < 1e9;
-            double dx[6], dpx[6], dz[6], dpz[6], ex[6], epx[6], ez[6], epz[6];
-            delta_weights(qx - flx, g.h, dx, dpx);
-            delta_weights(qz - flz, g.h, dz, dpz);
-            delta_weights_dxs(qx - flx, g.h, ex, epx);
-            delta_weights_dxs(qz - flz, g.h, ez, epz);
-            kx = ok ? (int)flx : 0;
-            kz = ok ? (int)flz : 0;
-            i0 = kx - 2;
-            j0 = kz - 2;
-            span = 6;
-            const double mxx = th[4], mxz = th[5], mzz = th[6];
-            for (int b = 0; b < 6; b++)
-                for (int a2 = 0; a2 < 6; a2++) {
-                    double vx = 0.0, vz = 0.0;
-                    if (p == 0) {
-                        vx = mxx * epx[a2] * dz[b] + mxz * ex[a2] * dpz[b];
-                        vz = mxz * epx[a2] * dz[b] + mzz * ex[a2] * dpz[b];
-                    } else if (p == 1) {
-                        vx = mxx * dpx[a2] * ez[b] + mxz * dx[a2] * epz[b];
-                        vz = mxz * dpx[a2] * ez[b] + mzz * dx[a2] * epz[b];
-                    } else if (p == 2 || p == 3) {
-                        vx = mxx * dpx[a2] * dz[b] + mxz * dx[a2] * dpz[b];
-                        vz = mxz * dpx[a2] * dz[b] + mzz * dx[a2] * dpz[b];
-                    } else if (p == 4) {
-                        vx = dpx[a2] * dz[b];
-                    } else if (p == 5) {
-                        vx = dx[a2] * dpz[b];
-                        vz = dpx[a2] * dz[b];
-                    } else {
-                        vz = dx[a2] * dpz[b];
-                    }
-                    w7x[b * kPatch + a2] = vx;
-                    w7z[b * kPatch + a2] = vz;
-                }
-        } else if (!diff || time_diff) {
-            ok = source_patch6(th, g.h, &kx, &kz, fx, fz);
-            i0 = kx - 2;
-            j0 = kz - 2;
-            span = 6;
-            for (int b = 0; b < 6; b++)
-                for (int a = 0; a < 6; a++) {
-                    w7x[b * kPatch + a] = fx[b * 6 + a];
-                    w7z[b * kPatch + a] = fz[b * 6 + a];
-                }
-        } else {
-            double gx[36], gz[36];
-            int kx2 = 0, kz2 = 0;
-            ok = source_patch6(tp, g.h, &kx, &kz, fx, fz) && source_patch6(tm, g.h, &kx2, &kz2, gx, gz);
-            const int kxm = min(kx, kx2), kzm = min(kz, kz2);
-            ok = ok && max(kx, kx2) - kxm <= 1 && max(kz, kz2) - kzm <= 1;
-            i0 = kxm - 2;
-            j0 = kzm - 2;
-            span = (kx != kx2 || kz != kz2) ? 7 : 6;
-            if (ok) {
-                const int ox = kx - kxm, oz = kz - kzm, ox2 = kx2 - kxm, oz2 = kz2 - kzm;
-                for (int b = 0; b < 6; b++)
-                    for (int a = 0; a < 6; a++) {
-                        w7x[(b + oz) * kPatch + a + ox] += fx[b * 6 + a];
-                        w7z[(b + oz) * kPatch + a + ox] += fz[b * 6 + a];
-                        w7x[(b + oz2) * kPatch + a + ox2] -= gx[b * 6 + a];
-                        w7z[(b + oz2) * kPatch + a + ox2] -= gz[b * 6 + a];
-                    }
+    // entry j of solve p's parameter vector
+    auto param = [&](int p, int j) {
+        return pairs && p > 0 && (p - 1) / 2 == j ? ((p - 1) & 1 ? thm[j] : thp[j]) : th[j];
+    };
+    // position (0 node, 1 +, 2 -) of solve p on an axis
+    auto position = [&](int p, int axis) { return pairs && p > 0 && (p - 1) / 2 == axis ? 1 + ((p - 1) & 1) : 0; };
+    if (blockIdx.y == 0) {
+        if (tid < 6) {
+            const int axis = tid / 3, v = tid % 3;
+            if (v == 0 || diff || pairs) {
+                const double q = (v == 0 ? th : v == 1 ? thp : thm)[axis] / g.h, fl = floor(q);
+                const bool ok = isfinite(q) && fabs(fl) < 1e9;
+                fin[axis][v] = ok;
+                cell[axis][v] = ok ? (int)fl : 0;
+                delta_weights(q - fl, g.h, W[axis][v][0], W[axis][v][1]);
+                if (sens) delta_weights_dxs(q - fl, g.h, W[axis][v][2], W[axis][v][3]);
             }
         }
-        ok = ok && i0 >= 1 && i0 + span - 1 <= g.nx - 2 && j0 >= 0 && j0 + span - 1 <= g.nz - 2;
-        corner[0] = ok ? i0 : -100;
-        corner[1] = ok ? j0 : -100;
-        corner[2] = ok;
-        src[s].i0 = corner[0];
-        src[s].j0 = corner[1];
-        src[s].ok = ok;
+        __syncthreads();
+        if (tid < per_node) {
+            const int p = tid;
+            int i0, j0, span = 6;   // span: 6 or 7 nodes of the patch actually used
+            bool ok;
+            if (diff && p != 2 && p != 3) {
+                const int px = p == 0, pz = p == 1;   // the axis that is perturbed has positions 1 and 2
+                const int xa = cell[0][px], xb = cell[0][2 * px], za = cell[1][pz], zb = cell[1][2 * pz];
+                ok = fin[0][px] && fin[0][2 * px] && fin[1][pz] && fin[1][2 * pz];
+                i0 = min(xa, xb) - 2;
+                j0 = min(za, zb) - 2;
+                ok = ok && max(xa, xb) - min(xa, xb) <= 1 && max(za, zb) - min(za, zb) <= 1;
+                if (xa != xb || za != zb) span = 7;
+            } else {
+                const int vx = position(p, 0), vz = position(p, 1);
+                ok = fin[0][vx] && fin[1][vz];
+                i0 = cell[0][vx] - 2;
+                j0 = cell[1][vz] - 2;
+            }
+            ok = ok && i0 >= 1 && i0 + span - 1 <= g.nx - 2 && j0 >= 0 && j0 + span - 1 <= g.nz - 2;
+            corner[p][0] = ok ? i0 : -100;
+            corner[p][1] = ok ? j0 : -100;
+            corner[p][2] = ok;
+            SourceDesc<real> &d = src[(size_t)node * per_node + p];
+            d.i0 = corner[p][0];
+            d.j0 = corner[p][1];
+            d.ok = ok;
+        }
+        __syncthreads();
+        for (int k = tid; k < per_node * kPatch * kPatch; k += blockDim.x) {
+            const int p = k / (kPatch * kPatch), e = k % (kPatch * kPatch), b = e / kPatch, a = e % kPatch;
+            double vx = 0.0, vz = 0.0;
+            // M grad(delta) of positions (px, pz) with moments m at support entry (bb, aa)
+            auto force = [&](int px, int pz, double mxx, double mxz, double mzz, int bb, int aa, double &fx, double &fz) {
+                fx = fz = 0.0;
+                if ((unsigned)aa >= 6u || (unsigned)bb >= 6u) return;
+                const double dx = W[0][px][0][aa], dpx = W[0][px][1][aa], dz = W[1][pz][0][bb], dpz = W[1][pz][1][bb];
+                fx = mxx * dpx * dz + mxz * dx * dpz;
+                fz = mxz * dpx * dz + mzz * dx * dpz;
+            };
+            if (sens) {
+                if (a < 6 && b < 6) {
+                    const double dx = W[0][0][0][a], dpx = W[0][0][1][a], ex = W[0][0][2][a], epx = W[0][0][3][a];
+                    const double dz = W[1][0][0][b], dpz = W[1][0][1][b], ez = W[1][0][2][b], epz = W[1][0][3][b];
+                    const double mxx = th[4], mxz = th[5], mzz = th[6];
+                    if (p == 0) {
+                        vx = mxx * epx * dz + mxz * ex * dpz;
+                        vz = mxz * epx * dz + mzz * ex * dpz;
+                    } else if (p == 1) {
+                        vx = mxx * dpx * ez + mxz * dx * epz;
+                        vz = mxz * dpx * ez + mzz * dx * epz;
+                    } else if (p == 2 || p == 3) {
+                        vx = mxx * dpx * dz + mxz * dx * dpz;
+                        vz = mxz * dpx * dz + mzz * dx * dpz;
+                    } else if (p == 4) {
+                        vx = dpx * dz;
+                    } else if (p == 5) {
+                        vx = dx * dpz;
+                        vz = dpx * dz;
+                    } else {
+                        vz = dx * dpz;
+                    }
+                }
+            } else if (diff && p != 2 && p != 3) {
+                const int px = p == 0, pz = p == 1;
+                const int xa = cell[0][px], xb = cell[0][2 * px], za = cell[1][pz], zb = cell[1][2 * pz];
+                if (corner[p][2]) {
+                    double gx, gz;
+                    force(px, pz, p == 4 ? thp[4] : th[4], p == 5 ? thp[5] : th[5], p == 6 ? thp[6] : th[6],
+                          b - (za - min(za, zb)), a - (xa - min(xa, xb)), vx, vz);
+                    force(2 * px, 2 * pz, p == 4 ? thm[4] : th[4], p == 5 ? thm[5] : th[5], p == 6 ? thm[6] : th[6],
+                          b - (zb - min(za, zb)), a - (xb - min(xa, xb)), gx, gz);
+                    vx = vx - gx;
+                    vz = vz - gz;
+                }
+            } else {
+                force(position(p, 0), position(p, 1), param(p, 4), param(p, 5), param(p, 6), b, a, vx, vz);
+            }
+            const int j = corner[p][1] + b;
+            const double rf = (corner[p][2] && j <= g.nz - 1) ? (double)rows[j].rf : 0.0;
+            SourceDesc<real> &d = src[(size_t)node * per_node + p];
+            d.wx[e] = (real)(vx * rf);
+            d.wz[e] = (real)(vz * rf);
+        }
+        for (int k = tid; k < per_node * kNT; k += blockDim.x)
+            theta_out[(size_t)node * per_node * kNT + k] = param(k / kNT, k % kNT);
     }
-    __syncthreads();
-    for (int k = threadIdx.x; k < kPatch * kPatch; k += blockDim.x) {
-        const int b = k / kPatch;
-        const int j = corner[1] + b;
-        const double rf = (corner[2] && j <= g.nz - 1) ? (double)rows[j].rf : 0.0;
-        src[s].wx[k] = (real)(w7x[k] * rf);
-        src[s].wz[k] = (real)(w7z[k] * rf);
-    }
-    for (int m = threadIdx.x; m < g.nsteps; m += blockDim.x) {
+    const double ts = th[2], ws = th[3];
+    real *out = stf + (size_t)node * per_node * g.nsteps;
+    for (int m = blockIdx.y * blockDim.x + tid; m < g.nsteps; m += gridDim.y * blockDim.x) {
         const double t = m * g.dt;
-        double v = time_diff ? stf_value(stf_kind, t, tp[2], tp[3]) - stf_value(stf_kind, t, tm[2], tm[3])
-                             : stf_value(stf_kind, t, th[2], th[3]);
-        // (sensitivity solves: Gaussian only, the host refuses them for any other kind)
-        if (time_kind == 1) v *= th[3] * th[3] * (t - th[2]);                 // dS/dt_s
-        if (time_kind == 2) v *= 1.0 / th[3] - th[3] * (t - th[2]) * (t - th[2]);   // dS/domega_s
-        stf[(size_t)s * g.nsteps + m] = (real)v;
+        const double S = stf_value(stf_kind, t, ts, ws);
+        double v2 = S, v3 = S;   // solves of t_s and omega_s: difference or derivative
+        if (sens) {   // (Gaussian only, the host refuses sensitivity solves for any other kind)
+            v2 *= ws * ws * (t - ts);                        // dS/dt_s
+            v3 *= 1.0 / ws - ws * (t - ts) * (t - ts);       // dS/domega_s
+        } else if (diff) {
+            v2 = stf_value(stf_kind, t, thp[2], ws) - stf_value(stf_kind, t, thm[2], ws);
+            v3 = stf_value(stf_kind, t, ts, thp[3]) - stf_value(stf_kind, t, ts, thm[3]);
+        }
+        for (int p = 0; p < per_node; p++) {
+            double v = S;
+            if (pairs) {
+                if (p == 5) v = stf_value(stf_kind, t, thp[2], ws);
+                if (p == 6) v = stf_value(stf_kind, t, thm[2], ws);
+                if (p == 7) v = stf_value(stf_kind, t, ts, thp[3]);
+                if (p == 8) v = stf_value(stf_kind, t, ts, thm[3]);
+            } else if (per_node == kND) {
+                if (p == 2) v = v2;
+                if (p == 3) v = v3;
+            }
+            out[(size_t)p * g.nsteps + m] = (real)v;
+        }
     }
 }
 
@@ -476,16 +489,18 @@ void launch_sources(const oed_ctx *ctx, const double *theta_nodes, int nnode, in
     const int sens = (per_node == kND && ctx->jac_mode == OED_JAC_SENSITIVITY) ? 1 : 0;
     FdStep st;
     for (int j = 0; j < kNT; j++) st.d[j] = step ? step[j] : 0.0;
-    const int nsolve = nnode * per_node;
-    if (nsolve <= 0) return;
+    if (nnode <= 0) return;
+    // few nodes: their time steps are spread over several blocks
+    const int parts = std::max(1, std::min((ctx->g.nsteps + 127) / 128, 304 / nnode));
+    const dim3 grid(nnode, parts);
     if (ctx->precision == OED_FP64)
-        k_sources<double><<<nsolve, 128, 0, s>>>(
-            theta_nodes, nsolve, per_node, sens, ctx->stf, st, ctx->g, (const RowCoef<double> *)ctx->d_rows,
-            (SourceDesc<double> *)ctx->d_src, (double *)ctx->d_stf, ctx->d_theta);
+        k_sources<double><<<grid, 128, 0, s>>>(theta_nodes, per_node, sens, ctx->stf, st, ctx->g,
+                                               (const RowCoef<double> *)ctx->d_rows, (SourceDesc<double> *)ctx->d_src,
+                                               (double *)ctx->d_stf, ctx->d_theta);
     else
-        k_sources<float><<<nsolve, 128, 0, s>>>(
-            theta_nodes, nsolve, per_node, sens, ctx->stf, st, ctx->g, (const RowCoef<float> *)ctx->d_rows,
-            (SourceDesc<float> *)ctx->d_src, (float *)ctx->d_stf, ctx->d_theta);
+        k_sources<float><<<grid, 128, 0, s>>>(theta_nodes, per_node, sens, ctx->stf, st, ctx->g,
+                                              (const RowCoef<float> *)ctx->d_rows, (SourceDesc<float> *)ctx->d_src,
+                                              (float *)ctx->d_stf, ctx->d_theta);
 }
 
 }  // namespace oed
