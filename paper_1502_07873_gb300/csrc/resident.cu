@@ -48,7 +48,7 @@ namespace oed {
 // two, four or five.
 constexpr int kResThreads = 640;
 constexpr int kResRegs = 96;
-constexpr int kResRegsHom = 88;   // homogeneous medium, several CTAs: 640 Gcell-upd/s on 401x201 (96: 629)
+constexpr int kResRegsHom = 96;   // homogeneous medium, several CTAs
 constexpr size_t kSmemPerSm = 228 * 1024;   // shared memory of an SM, 1 KB of it reserved per CTA
 
 struct ResArgs {
@@ -92,6 +92,18 @@ __device__ __forceinline__ unsigned remote_addr(unsigned local, unsigned rank)
     return r;
 }
 
+__device__ __forceinline__ float2 lds2(unsigned a)
+{
+    float2 v;
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ void sts2(unsigned a, float2 v)
+{
+    asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(v.x), "f"(v.y) : "memory");
+}
+
 __device__ __forceinline__ float2 ld_cluster2(unsigned addr)
 {
     float2 v;
@@ -103,48 +115,50 @@ __device__ __forceinline__ float2 ld_cluster2(unsigned addr)
 // columns' in the next sq: slot q of each half belongs to the column pair p = q - 1, so
 // the pair of a thread is (E[q], O[q]), its west column O[q-1] and its east column
 // E[q+1] -- four 64-bit loads at an 8-byte stride across the warp, no bank conflicts.
-// q points at the thread's even slot of the row.
-__device__ __forceinline__ float4 pair_at(const float2 *q, int sq)
+// Addresses are 32-bit shared ones: a is the thread's even slot of a row, so8 the bytes from
+// the even half to the odd one.
+__device__ __forceinline__ float4 pair_at(unsigned a, unsigned so8)
 {
-    const float2 e = q[0], o = q[sq];
+    const float2 e = lds2(a), o = lds2(a + so8);
     return make_float4(e.x, e.y, o.x, o.y);
 }
 
 // The pair's slots in the level being written (u^{m-1} in, u^{m+1} out), at per-thread
-// offsets offE (column c) and offO (column c + 1) from q: 0 and sq for interior pairs.  A
+// byte offsets offE (column c) and offO (column c + 1) from a: 0 and so8 for interior pairs.  A
 // side column (or the ghost column nx) is written by the edge warp, not by the march, so
 // its thread's slot is moved to a ghost slot that no thread reads (even slot 0, or slot
 // npair + 1 of either half): the march's stores stay unconditional.
-__device__ __forceinline__ float4 pair_at_n(const float2 *q, int offE, int offO)
+__device__ __forceinline__ float4 pair_at_n(unsigned a, int offE, int offO)
 {
-    const float2 e = q[offE], o = q[offO];
+    const float2 e = lds2(a + offE), o = lds2(a + offO);
     return make_float4(e.x, e.y, o.x, o.y);
 }
 
-__device__ __forceinline__ void pair_put_n(float2 *q, int offE, int offO, float4 u)
+__device__ __forceinline__ void pair_put_n(unsigned a, int offE, int offO, float4 u)
 {
-    q[offE] = make_float2(u.x, u.y);
-    q[offO] = make_float2(u.z, u.w);
+    sts2(a + offE, make_float2(u.x, u.y));
+    sts2(a + offO, make_float2(u.z, u.w));
 }
 
-__device__ __forceinline__ void load_row(const float2 *q, int sq, Row2P &r)
+__device__ __forceinline__ void load_row(unsigned a, unsigned so8, Row2P &r)
 {
-    row_fromP(q[sq - 1], pair_at(q, sq), q[1], r);
+    const float4 m = pair_at(a, so8);
+    row_fromP(lds2(a + so8 - 8u), m, lds2(a + 8u), r);
 }
 
 // the same slots of a row in CTA `nb` of the cluster
-__device__ __forceinline__ float4 pair_at_remote(const float2 *q, int sq, unsigned nb)
+__device__ __forceinline__ float4 pair_at_remote(unsigned a, unsigned so8, unsigned nb)
 {
-    const unsigned b = remote_addr(smem_addr(q), nb);
-    const float2 e = ld_cluster2(b), o = ld_cluster2(b + 8u * (unsigned)sq);
+    const unsigned b = remote_addr(a, nb);
+    const float2 e = ld_cluster2(b), o = ld_cluster2(b + so8);
     return make_float4(e.x, e.y, o.x, o.y);
 }
 
-__device__ __forceinline__ void load_row_remote(const float2 *q, int sq, unsigned nb, Row2P &r)
+__device__ __forceinline__ void load_row_remote(unsigned a, unsigned so8, unsigned nb, Row2P &r)
 {
-    const unsigned b = remote_addr(smem_addr(q), nb);
-    const float2 e = ld_cluster2(b), o = ld_cluster2(b + 8u * (unsigned)sq);
-    row_fromP(ld_cluster2(b + 8u * (unsigned)(sq - 1)), make_float4(e.x, e.y, o.x, o.y), ld_cluster2(b + 8u), r);
+    const unsigned b = remote_addr(a, nb);
+    const float2 e = ld_cluster2(b), o = ld_cluster2(b + so8);
+    row_fromP(ld_cluster2(b + so8 - 8u), make_float4(e.x, e.y, o.x, o.y), ld_cluster2(b + 8u), r);
 }
 
 // float offset of node (column i, component comp) within a shared row
@@ -169,6 +183,7 @@ __global__ void __maxnreg__(HOM && !ONE ? kResRegsHom : kResRegs) k_resident(Res
     const int RS = 2 * sq;    // float2 slots per row
     float2 *A = reinterpret_cast<float2 *>(smem4), *B = A + R * RS;
     KP *coef = reinterpret_cast<KP *>(smem4 + 2 * lvl);
+    const unsigned level0 = smem_addr(A), lvl16 = 16u * (unsigned)lvl;   // shared address of level A; B is lvl16 on
     const int tid = threadIdx.x;
     const int nthr = blockDim.x;
 
@@ -189,9 +204,11 @@ __global__ void __maxnreg__(HOM && !ONE ? kResRegsHom : kResRegs) k_resident(Res
     const int seg = tid / a.npair;
     const bool active = !edge && seg < a.nseg;
     const int kind = (c == 0 ? 1 : 0) | (c + 1 == g.nx - 1 ? 2 : 0) | (c == g.nx - 1 ? 4 : 0);
-    const int offE = (kind & 1) ? -1 : ((kind & 4) ? 1 : 0);
-    const int offO = a.sq + ((kind & 6) ? 1 : 0);
+    const unsigned so8 = 8u * (unsigned)sq, rs8 = 8u * (unsigned)RS;   // bytes: half row, row
+    const int offE = (kind & 1) ? -8 : ((kind & 4) ? 8 : 0);
+    const int offO = (int)so8 + ((kind & 6) ? 8 : 0);
     const int l0 = seg * a.rps;
+    const unsigned slot0 = level0 + 8u * (unsigned)(l0 * RS + p + 1);
     const int l1 = min(l0 + a.rps, nrows);
     const bool top = (j0 + l0 == 0);
     const SourceDesc<float> *sd = a.src + s;
@@ -226,8 +243,8 @@ __global__ void __maxnreg__(HOM && !ONE ? kResRegsHom : kResRegs) k_resident(Res
     if (!ONE) cluster_barrier();
 
     for (int m = 0; m < g.nsteps; m++) {
-        const float2 *cur = ((m & 1) ? B : A) + p + 1;   // this thread's even slot in row 0
-        float2 *nxt = ((m & 1) ? A : B) + p + 1;
+        // this thread's even slot in its segment's first row
+        const unsigned cur = slot0 + ((m & 1) ? lvl16 : 0u), nxt = slot0 + ((m & 1) ? 0u : lvl16);
         if (edge) {
             const int e = tid - a.nmarch;
             const float *cf = reinterpret_cast<const float *>((m & 1) ? B : A);   // u^m
@@ -252,59 +269,71 @@ __global__ void __maxnreg__(HOM && !ONE ? kResRegsHom : kResRegs) k_resident(Res
         if (active && l0 < l1) {
             Row2P rn, rc, rs;
             int l = l0;
-            load_row(cur + l * RS, sq, rc);
+            load_row(cur, so8, rc);
+            unsigned cl = cur, nl = nxt;   // the even slot in row l of u^m, of u^{m+1}
             if (top) {   // surface row: no north differences, cross terms on the row itself
                 if (ONE || l + 1 < nrows)
-                    load_row(cur + (l + 1) * RS, sq, rs);
+                    load_row(cur + rs8, so8, rs);
                 else   // a one-row slab
-                    load_row_remote(cur, sq, rank + 1, rs);
+                    load_row_remote(cur, so8, rank + 1, rs);
                 southP(rc, rs);
                 Row2P nt = rc;
                 nt.va = nt.vb = make_float2(0.0f, 0.0f);
-                float2 *o = nxt + l * RS;
-                float4 u = pair_at_n(o, offE, offO);
+                float4 u = pair_at_n(nxt, offE, offO);
                 const KP K = coef[l];
                 pair_updateP(K, nt, rc, rs, u);
-                pair_put_n(o, offE, offO, u);
+                pair_put_n(nxt, offE, offO, u);
                 rn = rc;
                 rc = rs;
                 l++;
+                cl += rs8;
+                nl += rs8;
             } else {
                 if (ONE || l > 0)
-                    load_row(cur + (l - 1) * RS, sq, rn);
+                    load_row(cur - rs8, so8, rn);
                 else
-                    load_row_remote(cur + (R - 1) * RS, sq, rank - 1, rn);
+                    load_row_remote(cur + (R - 1) * rs8, so8, rank - 1, rn);
                 southP(rn, rc);
             }
             // rows whose south neighbour is a local row and that are not the bottom row:
             // unrolled by three with the three window rows taking turns
             const int lstop = min(l1, nrows - 1);
             if (l < lstop) {
-                // the loads of the next row are issued before the update of this one
-                const float2 *sp = cur + (l + 1) * RS;
-                float2 *o = nxt + l * RS;
+                // Four shared addresses move down with the march: the even and odd slots of the row
+                // to fetch, and of the row whose u^{m-1} is fetched with it and that is stored next
+                unsigned pe = cl + rs8, po = pe + so8, we = nl + offE, wo = nl + offO;
                 const KP *cf = coef + l;
-                float4 pm = pair_at(sp, sq), pu = pair_at_n(o, offE, offO);
-                float2 pw = sp[sq - 1];
-                float2 pe = sp[1];
+                // the loads of the next row are issued before the update of this one
+                float4 pm, pu;
+                float2 pw, px;
+                auto fetch = [&] {
+                    const float2 e = lds2(pe), o = lds2(po);
+                    pm = make_float4(e.x, e.y, o.x, o.y);
+                    pw = lds2(po - 8u);
+                    px = lds2(pe + 8u);
+                    const float2 a0 = lds2(we), b0 = lds2(wo);
+                    pu = make_float4(a0.x, a0.y, b0.x, b0.y);
+                };
+                fetch();
                 // pf: a row below the south row exists, prefetch it (every row but the last)
                 // unifK: each lane's march rows share its K0 (no coefficient loads)
                 auto march = [&](auto unifK) {
                     auto row = [&](auto pf, const Row2P &wn, Row2P &wc, Row2P &ws) {
-                        row_fromP(pw, pm, pe, ws);
+                        row_fromP(pw, pm, px, ws);
                         float4 u = pu;
+                        const unsigned se = we, so = wo;
                         if constexpr (decltype(pf)::value) {
-                            sp += RS;
-                            pm = pair_at(sp, sq);
-                            pw = sp[sq - 1];
-                            pe = sp[1];
-                            pu = pair_at_n(o + RS, offE, offO);
+                            pe += rs8;
+                            po += rs8;
+                            we += rs8;
+                            wo += rs8;
+                            fetch();
                         }
                         southP(wc, ws);
                         const KP K = decltype(unifK)::value ? K0 : *cf;
                         pair_updateP(K, wn, wc, ws, u);
-                        pair_put_n(o, offE, offO, u);
-                        o += RS;
+                        sts2(se, make_float2(u.x, u.y));
+                        sts2(so, make_float2(u.z, u.w));
                         cf++;
                     };
                     const std::true_type P{};
@@ -343,22 +372,20 @@ __global__ void __maxnreg__(HOM && !ONE ? kResRegsHom : kResRegs) k_resident(Res
             }
             // what is left: a last interior row whose south neighbour sits in CTA rank+1,
             // or the absorbing bottom row
-            for (; l < l1; l++) {
+            if (l < l1) {
+                const unsigned lr = (unsigned)(l - l0) * rs8;
                 const KP K = coef[l];
-                float2 *o = nxt + l * RS;
-                float4 u = pair_at_n(o, offE, offO);
+                float4 u = pair_at_n(nxt + lr, offE, offO);
                 if (ONE || j0 + l == g.nz - 1) {
-                    const float4 nv = ONE || l > 0 ? pair_at(cur + (l - 1) * RS, sq)
-                                            : pair_at_remote(cur + (R - 1) * RS, sq, rank - 1);
+                    const float4 nv = ONE || l > 0 ? pair_at(cur + lr - rs8, so8)
+                                                   : pair_at_remote(cur + (R - 1) * rs8, so8, rank - 1);
                     absorbingP(K.c, nv, rc, true, 0, u);
                 } else {
-                    load_row_remote(cur, sq, rank + 1, rs);
+                    load_row_remote(cur - (unsigned)l0 * rs8, so8, rank + 1, rs);
                     southP(rc, rs);
                     pair_updateP(K, rn, rc, rs, u);
                 }
-                pair_put_n(o, offE, offO, u);
-                rn = rc;
-                rc = rs;
+                pair_put_n(nxt + lr, offE, offO, u);
             }
         }
         if (patch_warp)
