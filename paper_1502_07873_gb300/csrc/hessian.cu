@@ -8,21 +8,37 @@
 // in FP64 from the +/- pair, J_j = (g_{+j} - g_{-j}) / (2 d_j).  Difference form
 // (7 solves per node): solve j already holds g_{+j} - g_{-j} (its forcing is the
 // FP64 difference of the two forcings), so J_j = g_j / (2 d_j).  The 28 unique
-// products are accumulated in FP64.  One block handles one
+// products of the differences are accumulated in FP64, the factors 1 / (4 d_x d_y) applied to
+// the sums (the FP64 pipe bounds the kernel: 28 slots a row in the difference form, 35 in the
+// pairs form, against 42 and 56 with scaled and converted entries; 1024 nodes x 321 levels x
+// 91 receivers 4.06 ms against 4.96).  One block handles one
 // node and one time sub-segment; its threads walk the flattened (m, r, c) rows so
 // that a warp reads consecutive (r, c) of the same level (coalesced), and each
 // thread keeps a single (r, c) so its 28 partial sums belong to one receiver.
+#include <algorithm>
+
 #include "oed_internal.cuh"
 
 namespace oed {
 
 struct HArgs {
-    double inv2d[kNT];      // 1 / (2 d_j)
+    double scale[28];       // 1 / (4 d_x d_y) of the upper triangle's entries
     int sub_m0[16];         // sub-segment level ranges [m0, m1)
     int sub_m1[16];
     int win_sub_end[16];    // window w ends with sub-segment win_sub_end[w] - 1
     int nsub;
 };
+
+// The exact FP64 value of an FP32 one in integer operations, which are free beside the FP64
+// pipe (a conversion instruction takes a slot of it)
+__device__ __forceinline__ double widen(float x)
+{
+    const unsigned b = __float_as_uint(x), m = b & 0x7fffffffu;
+    if (m - 1u < 0x007fffffu || m >= 0x7f800000u) return (double)x;   // subnormal, infinite, NaN
+    const unsigned hi = m ? (m >> 3) + 0x38000000u : 0u;
+    return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)(b << 29));
+}
+__device__ __forceinline__ double widen(double x) { return x; }
 
 template <typename real, bool DIFF>
 __global__ void __launch_bounds__(512) k_hsub(const real *__restrict__ trace, Geometry g,
@@ -45,11 +61,10 @@ __global__ void __launch_bounds__(512) k_hsub(const real *__restrict__ trace, Ge
 #pragma unroll
             for (int j = 0; j < kNT; j++) {
                 if (DIFF) {
-                    J[j] = (double)base[(size_t)j * per_solve + off] * a.inv2d[j];
+                    J[j] = widen(base[(size_t)j * per_solve + off]);
                 } else {
-                    const double gp = (double)base[(size_t)(1 + 2 * j) * per_solve + off];
-                    const double gm = (double)base[(size_t)(2 + 2 * j) * per_solve + off];
-                    J[j] = (gp - gm) * a.inv2d[j];
+                    J[j] = widen(base[(size_t)(1 + 2 * j) * per_solve + off]) -
+                           widen(base[(size_t)(2 + 2 * j) * per_solve + off]);
                 }
             }
             int k = 0;
@@ -110,7 +125,7 @@ __global__ void k_hcombine(const double *__restrict__ hsub, Geometry g, double s
             run += hsub[(((size_t)node * nsub + sub) * nrec + r) * 28 + k];
             while (next < nwin && a.win_sub_end[next] == sub + 1) {
                 if (H_rec)
-                    H_rec[(((size_t)node * nrec + r) * nwin + next) * 28 + k] = ok == 1 ? s2 * run : nan;
+                    H_rec[(((size_t)node * nrec + r) * nwin + next) * 28 + k] = ok == 1 ? s2 * a.scale[k] * run : nan;
                 next++;
             }
         }
@@ -129,7 +144,7 @@ __global__ void k_hcombine(const double *__restrict__ hsub, Geometry g, double s
         const int x = threadIdx.x / 7, y = threadIdx.x % 7;
         const int a0 = x < y ? x : y, b0 = x < y ? y : x;
         const int k = a0 * 7 - a0 * (a0 - 1) / 2 + (b0 - a0);
-        H[(size_t)node * 49 + threadIdx.x] = ok == 1 ? s2 * tot[k] : nan;
+        H[(size_t)node * 49 + threadIdx.x] = ok == 1 ? s2 * a.scale[k] * tot[k] : nan;
     }
     if (threadIdx.x == 0 && status) status[node] = ok == 1 ? 0 : (ok < 0 ? OED_ETIMEOUT : OED_EINVAL);
 }
@@ -141,11 +156,16 @@ void launch_hessian(const oed_ctx *ctx, int nnode, const double *inv2d, double s
                     double *H_rec, int *status, cudaStream_t st)
 {
     // Split the level range into at most 16 sub-segments that respect the window
-    // boundaries seg_end[0..nseg) (seg_end[nseg-1] = nlev), enough for >= ~4 blocks per SM.
+    // boundaries seg_end[0..nseg) (seg_end[nseg-1] = nlev), to spread few nodes over the SMs.
     const Geometry &g = ctx->g;
     HArgs a;
-    for (int j = 0; j < kNT; j++) a.inv2d[j] = inv2d[j];
-    int want = 16;
+    for (int x = 0, k = 0; x < kNT; x++)
+        for (int y = x; y < kNT; y++) a.scale[k++] = inv2d[x] * inv2d[y];
+    // Shorter ones of under eight rows a thread spend more on their sums than on their rows (the
+    // paper's 51 levels at two receivers: 0.37 ms for 2048 nodes in sixteen, 0.05 in one).  The split
+    // depends on the problem alone, so that results do not depend on the chunk.
+    const int lanes = hsub_threads(g.nrec) / (2 * g.nrec);
+    const int want = std::max(1, std::min(16, g.nlev / (8 * lanes)));
     int per = want / nseg;
     if (per < 1) per = 1;
     int nsub = 0;
