@@ -20,6 +20,8 @@
 //   acc[s][c][node] += lambda^m(node, c) * S_s(t_{m-1}),   s = S, S_t, S_w, S_tt, S_tw, S_ww,
 // from which the forcing's first and second parameter derivatives give the cost
 // gradient and H_II (source.cu, k_hii_combine).
+#include <algorithm>
+
 #include "oed_internal.cuh"
 
 namespace oed {
@@ -139,6 +141,111 @@ __global__ void __launch_bounds__(256) k_adjoint_step(AdjArgs<real> a)
     oz[o] = sz;
 }
 
+// The same in FP64, where the pipe (two lanes per clock and SM) is the bound and only its
+// issue slots count: 16 per node and a little per row segment, against 37 with a branch per
+// neighbour and the centre coefficients formed anew at every node.  A thread takes a column's
+// segment of up to ZS rows, threads are packed densely over solves, segments and columns, the
+// east - west differences of a row serve the rows above and below it, and the boundary nodes
+// take the slots of the interior with selected operands: a neighbour that is no interior node
+// enters as zero, the absorbing nodes' terms in the place of the missing neighbour's.
+struct AdjRow {
+    double w[2], c[2], e[2];   // lambda at i-1, i, i+1 (u_x, then u_z)
+    double d[2];               // west - east, interior nodes only
+};
+
+template <int ZS>
+__global__ void __launch_bounds__(128) k_adjoint64(AdjArgs<double> a, int nseg, unsigned nthr)
+{
+    const Geometry &g = a.g;
+    const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= nthr) return;
+    const unsigned per = (unsigned)g.nx * (unsigned)nseg;
+    const int s = (int)(t / per);
+    const unsigned q = t - (unsigned)s * per;
+    const int seg = (int)(q / (unsigned)g.nx), i = (int)(q - (unsigned)seg * (unsigned)g.nx);
+    const int j0 = (int)((long long)g.nz * seg / nseg), j1 = (int)((long long)g.nz * (seg + 1) / nseg);
+    const double *__restrict__ cur = a.cur + (size_t)s * g.solve_stride + i;
+    double *__restrict__ nxt = a.nxt + (size_t)s * g.solve_stride + i;
+    const bool side = i == 0 || i == g.nx - 1, hasw = i > 0, hase = i < g.nx - 1;
+    const bool inw = i - 1 >= 1, ine = i + 1 <= g.nx - 2;   // the west / east column holds interior nodes
+    auto load = [&](int j, AdjRow &r) {
+        const bool in = j >= 0 && j < g.nz, rowin = in && j <= g.nz - 2;
+        const size_t o = (size_t)(in ? j : 0) * g.xp;
+#pragma unroll
+        for (int k = 0; k < 2; k++) {
+            const double *u = cur + k * g.comp_stride + o;
+            r.c[k] = in ? __ldg(u) : 0.0;
+            r.w[k] = in && hasw ? __ldg(u - 1) : 0.0;
+            r.e[k] = in && hase ? __ldg(u + 1) : 0.0;
+            r.d[k] = (rowin && inw ? r.w[k] : 0.0) - (rowin && ine ? r.e[k] : 0.0);
+        }
+    };
+    AdjRow n, c, so;
+    load(j0 - 1, n);
+    load(j0, c);
+#pragma unroll
+    for (int k0 = 0; k0 < ZS; k0++) {
+        const int j = j0 + k0;
+        if (j >= j1) break;
+        const bool bottom = j == g.nz - 1, inner = !side && !bottom;
+        const size_t o = (size_t)j * g.xp;
+        const FacCoef<double> K = a.fac[j], Kn = a.fac[j > 0 ? j - 1 : 0], Ks = a.fac[bottom ? j : j + 1];
+        const double ox = __ldcs(nxt + o), oz = __ldcs(nxt + g.comp_stride + o);
+        load(j + 1, so);
+        // the node's own update and E^T lambda^{m+2}; pad0 .. pad3: centre coefficients of u_x, u_z
+        // and 1 - c_p, 1 - c_s
+        double sx = fma(side ? K.pad2 : (bottom ? K.pad3 : K.pad0), c.c[0], inner ? -ox : 0.0);
+        double sz = fma(side ? K.pad3 : (bottom ? K.pad2 : K.pad1), c.c[1], inner ? -oz : 0.0);
+        // west and east neighbours on the row, or the absorbing side node whose inward neighbour this is
+        const double axx = bottom ? 0.0 : K.axx, azx = bottom ? 0.0 : K.azx;
+        sx = fma(i == 1 ? K.cp : (inw ? axx : 0.0), c.w[0], sx);
+        sz = fma(i == 1 ? K.cs : (inw ? azx : 0.0), c.w[1], sz);
+        sx = fma(i == g.nx - 2 ? K.cp : (ine ? axx : 0.0), c.e[0], sx);
+        sz = fma(i == g.nx - 2 ? K.cs : (ine ? azx : 0.0), c.e[1], sz);
+        // the row above (this node is its south) and the row below (its north, or the absorbing bottom)
+        const bool last = j == g.nz - 2;
+        sx = fma(side ? 0.0 : Kn.axzp, n.c[0], sx);
+        sz = fma(side ? 0.0 : Kn.azzp, n.c[1], sz);
+        sx = fma(side ? 0.0 : (last ? Ks.cs : -Ks.naxzm), so.c[0], sx);
+        sz = fma(side ? 0.0 : (last ? Ks.cp : -Ks.nazzm), so.c[1], sz);
+        // cross terms: u_x(i,j) enters the u_z update of the diagonal neighbours and vice versa
+        sx = fma(Kn.pz, n.d[1], sx);
+        sz = fma(Kn.px, n.d[0], sz);
+        sx = fma(Ks.nqz, so.d[1], sx);
+        sz = fma(Ks.nqx, so.d[0], sz);
+        if (j == 0) {   // the surface row's cross terms read its own row
+            sx = fma(K.nqz, c.d[1], sx);
+            sz = fma(K.nqx, c.d[0], sz);
+        }
+        nxt[o] = sx;
+        nxt[g.comp_stride + o] = sz;
+        n = c;
+        c = so;
+    }
+}
+
+static void adjoint_step(const AdjArgs<float> &a, int nsolve, cudaStream_t st)
+{
+    const dim3 blk(32, 8, 1), grd((a.g.nx + 31) / 32, (a.g.nz + 7) / 8, nsolve);
+    k_adjoint_step<float><<<grd, blk, 0, st>>>(a);
+}
+
+static void adjoint_step(const AdjArgs<double> &a, int nsolve, cudaStream_t st)
+{
+    constexpr int ZS = 4;   // 8 and 12 measured equal on 256 and 1000 solves of 101x76
+    const int nseg = segments64((long long)a.g.nx * nsolve, a.g.nz, ZS, 16.0, 8.0);
+    const long long per = (long long)a.g.nx * nseg;
+    const int most = (int)std::max(1LL, std::min((long long)nsolve, (1LL << 31) / per));   // 32-bit thread numbers
+    for (int s0 = 0; s0 < nsolve; s0 += most) {
+        const int ns = std::min(most, nsolve - s0);
+        AdjArgs<double> b = a;
+        b.cur += (size_t)s0 * a.g.solve_stride;
+        b.nxt += (size_t)s0 * a.g.solve_stride;
+        const unsigned nthr = (unsigned)(per * ns);
+        k_adjoint64<ZS><<<(nthr + 63) / 64, 64, 0, st>>>(b, nseg, nthr);
+    }
+}
+
 // S and its first and second derivatives in (t_s, omega_s): tau = t - t_s,
 // L = log S, dL/dt_s = w^2 tau, dL/dw = 1/w - w tau^2, d2L/dt_s2 = -w^2,
 // d2L/dt_s dw = 2 w tau, d2L/dw2 = -1/w^2 - tau^2, d2S = S (dL dL + d2L).
@@ -224,13 +331,12 @@ static void adjoint_impl(const oed_ctx *ctx, int nsolve, const double *y, double
     AdjArgs<real> a;
     a.fac = (const FacCoef<real> *)ctx->d_fac;
     a.g = g;
-    const dim3 blk(32, 8, 1), grd((g.nx + 31) / 32, (g.nz + 7) / 8, nsolve);
     real *A = (real *)ctx->d_u0, *B = (real *)ctx->d_u1;
     for (int m = g.nsteps; m >= 1; m--) {
         const int k = g.nsteps - m;
         a.cur = (k & 1) ? B : A;   // lambda^{m+1}
         a.nxt = (k & 1) ? A : B;   // lambda^{m+2} -> lambda^m
-        k_adjoint_step<real><<<grd, blk, 0, st>>>(a);
+        adjoint_step(a, nsolve, st);
         k_adjoint_post<real><<<nsolve, 128, 0, st>>>(a.nxt, w, ctx->d_rec, (const SourceDesc<real> *)ctx->d_src,
                                                      ctx->d_theta, acc, g, m);
     }

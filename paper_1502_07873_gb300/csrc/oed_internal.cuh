@@ -167,6 +167,8 @@ void launch_trace_to_f64(const oed_ctx *ctx, int nsolve, double *g, cudaStream_t
 void launch_step_probe(const oed_ctx *ctx, int nsolve, int nrep, cudaStream_t st, cudaEvent_t ev0,
                        cudaEvent_t ev1);
 
+int segments64(long long columns, int nz, int zs, double per, double once);   // FP64 row segments
+
 // stream_tma.cu
 bool tma_supported(const oed_ctx *ctx);
 int tma_prepare(oed_ctx *ctx);

@@ -347,7 +347,11 @@ __global__ void k_rows(Geometry g, int nlayers, const double *__restrict__ lay,
     q.axx = (real)f.axx; q.axzp = (real)f.axzp; q.naxzm = (real)f.naxzm; q.px = (real)f.px;
     q.nqx = (real)f.nqx; q.azx = (real)f.azx; q.azzp = (real)f.azzp; q.nazzm = (real)f.nazzm;
     q.pz = (real)f.pz; q.nqz = (real)f.nqz; q.cp = (real)c.cp; q.cs = (real)c.cs;
-    q.pad0 = q.pad1 = q.pad2 = q.pad3 = (real)0;
+    // for the dual problem: the centre coefficients of B and those of the absorbing nodes
+    q.pad0 = (real)2 - (real)2 * q.axx - q.axzp + q.naxzm;
+    q.pad1 = (real)2 - (real)2 * q.azx - q.azzp + q.nazzm;
+    q.pad2 = (real)1 - q.cp;
+    q.pad3 = (real)1 - q.cs;
     fac[j] = q;
 }
 

@@ -22,6 +22,7 @@
 // The same launch gathers the receiver samples of level m from its input u^m
 // (Eq. forward_model), so the seismograms need no extra pass over the field.
 #include <algorithm>
+#include <cmath>
 
 #include "stencil_cell.cuh"
 
@@ -268,6 +269,26 @@ __global__ void k_gather(const real *__restrict__ cur, real *__restrict__ trace,
         tr[q] = (q & 1 ? cz : cx)[rec[q >> 1]];
 }
 
+// Row segments for the FP64 kernels, columns of which (over all solves) take a thread each:
+// up to zs rows a segment, shorter where that spreads the columns over more of the schedulers
+// (four per SM, each with its own FP64 pipe).  A segment of r rows takes per r + once issue
+// slots, and the warps go round the schedulers.
+int segments64(long long columns, int nz, int zs, double per, double once)
+{
+    constexpr double kPipes = 4 * 152;
+    int best = (nz + zs - 1) / zs;
+    double least = 0.0;
+    for (int r = zs; r >= 1; r--) {
+        const int nseg = (nz + r - 1) / r;
+        const double cost = std::ceil((double)columns * nseg / 32.0 / kPipes) * (per * ((nz + nseg - 1) / nseg) + once);
+        if (r == zs || cost < least) {
+            least = cost;
+            best = nseg;
+        }
+    }
+    return best;
+}
+
 // One step of nsolve solves with the context's launch shape.
 template <typename real, int ZS>
 static void launch_one(const oed_ctx *ctx, int nsolve, const StepArgs<real> &a, cudaStream_t st)
@@ -275,7 +296,7 @@ static void launch_one(const oed_ctx *ctx, int nsolve, const StepArgs<real> &a, 
     const Geometry &g = ctx->g;
     const int wz = ctx->tune.wz;
     if constexpr (sizeof(real) == 8) {
-        const int npair = (g.nx + 1) / 2, nseg = (g.nz + ZS - 1) / ZS;
+        const int npair = (g.nx + 1) / 2, nseg = segments64((long long)npair * nsolve, g.nz, ZS, 23.0, 12.0);
         const long long per = (long long)npair * nseg;
         // 32-bit thread numbers: a batch past them goes in several launches
         const int most = (int)std::max(1LL, std::min((long long)nsolve, (1LL << 31) / per));
