@@ -4,9 +4,7 @@
 //
 // CTA r of a cluster of C owns rows [r R, min((r+1) R, nz)) of the grid, both
 // components and both time levels, in its shared memory:
-//     A, B : [R][npair + 2] float4,   coef : [R] KP (FacCoef in (x, z) pairs),   the solve's 2 x 49
-//     source weights (kept on chip: read from global memory every step they put an L1
-//     round trip on the critical path of the warps that own the patch columns)
+//     A, B : [R][npair + 2] float4,   coef : [R] KP (FacCoef in (x, z) pairs)
 // A row stores the even columns' (x, z) in sq = npair + 2 float2 slots, then the odd
 // columns' in sq more; slot q of each half belongs to the column pair p = q - 1, and
 // slots 0 and npair + 1 (columns -2, -1, nx.., and column nx when nx is odd) are zero
@@ -48,7 +46,7 @@ namespace oed {
 // two, four or five.
 constexpr int kResThreads = 640;
 constexpr int kResRegs = 96;
-constexpr int kResRegsHom = 96;   // homogeneous medium, several CTAs
+constexpr int kEdgeRec = 6;   // receiver offsets a lane of the edge warp keeps (96 receivers)
 constexpr size_t kSmemPerSm = 228 * 1024;   // shared memory of an SM, 1 KB of it reserved per CTA
 
 struct ResArgs {
@@ -77,6 +75,16 @@ __device__ __forceinline__ void cluster_barrier()
 {
     asm volatile("barrier.cluster.arrive.release.aligned;\n"
                  "barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+}
+
+// The end of a step: the edge warp and the march warps reach it from loops of their own
+template <bool ONE>
+__device__ __forceinline__ void step_barrier()
+{
+    if (ONE)
+        asm volatile("barrier.sync.aligned 0;" ::: "memory");
+    else
+        cluster_barrier();
 }
 
 // shared::cta address of a local pointer, and its image in CTA `rank` of the cluster
@@ -170,7 +178,7 @@ __device__ __forceinline__ int node_off(int i, int comp, int sq)
 // HOM: the medium is homogeneous, so every march row has the coefficients of row 1.
 // ONE: clusters of one CTA, no remote rows and a CTA barrier in place of the cluster's.
 template <bool HOM, bool ONE>
-__global__ void __maxnreg__(HOM && !ONE ? kResRegsHom : kResRegs) k_resident(ResArgs a)
+__global__ void __maxnreg__(kResRegs) k_resident(ResArgs a)
 {
     extern __shared__ float4 smem4[];
     const Geometry &g = a.g;
@@ -189,9 +197,6 @@ __global__ void __maxnreg__(HOM && !ONE ? kResRegsHom : kResRegs) k_resident(Res
 
     for (int k = tid; k < 2 * lvl; k += nthr) smem4[k] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     for (int k = tid; k < nrows; k += nthr) coef[k] = pack_coef(a.fac[j0 + k]);
-    float *sw = reinterpret_cast<float *>(coef + R);   // this solve's source weights, x then z
-    for (int k = tid; k < 2 * kPatch * kPatch; k += nthr)
-        sw[k] = k < kPatch * kPatch ? a.src[blockIdx.y].wx[k] : a.src[blockIdx.y].wz[k - kPatch * kPatch];
 
     // march threads are packed densely over (segment, pair): a warp may straddle two
     // segments.  The last warp (the edge warp) takes the absorbing side columns, which
@@ -242,20 +247,46 @@ __global__ void __maxnreg__(HOM && !ONE ? kResRegsHom : kResRegs) k_resident(Res
     const int npw = __syncthreads_count(patch_warp && (tid & 31) == 0);
     if (!ONE) cluster_barrier();
 
-    for (int m = 0; m < g.nsteps; m++) {
-        // this thread's even slot in its segment's first row
-        const unsigned cur = slot0 + ((m & 1) ? lvl16 : 0u), nxt = slot0 + ((m & 1) ? 0u : lvl16);
-        if (edge) {
-            const int e = tid - a.nmarch;
+    if (edge) {
+        // What the edge warp needs of a step beside u^m it holds in registers: on the step's
+        // critical path (the source term comes last, behind the march warps that own the patch)
+        // stand one wait, one shared load, one fma and one store.
+        const int e = tid - a.nmarch;
+        int ro[kEdgeRec];
+#pragma unroll
+        for (int k = 0; k < kEdgeRec; k++) {
+            const int q = e + 32 * k;
+            ro[k] = rank == 0 && q < 2 * g.nrec ? node_off(a.rec[q >> 1], q & 1, sq) : -1;
+        }
+        constexpr int kNodes = (kPatch * kPatch + 31) / 32;
+        int po[kNodes];
+        float wx[kNodes], wz[kNodes];
+#pragma unroll
+        for (int k = 0; k < kNodes; k++) {
+            const int q = e + 32 * k, bb = q / kPatch, ai = q - bb * kPatch, j = sj + bb;
+            po[k] = -1;
+            if (q < kPatch * kPatch && j >= srow0 && j < srow1) {
+                po[k] = (j - j0) * RS * 2 + node_off(si0 + ai, 0, sq);
+                wx[k] = sd->wx[q];
+                wz[k] = sd->wz[q];
+            }
+        }
+        const int oL = node_off(0, 0, sq), oL1 = node_off(1, 0, sq);
+        const int oR = node_off(g.nx - 1, 0, sq), oR1 = node_off(g.nx - 2, 0, sq);
+        float S = stf[0];
+        for (int m = 0; m < g.nsteps; m++) {
             const float *cf = reinterpret_cast<const float *>((m & 1) ? B : A);   // u^m
             float *nf = reinterpret_cast<float *>((m & 1) ? A : B);               // u^{m+1}
+            const float Sn = m + 1 < g.nsteps ? stf[m + 1] : 0.0f;
+            float *tr = trace + (size_t)m * g.nrec * 2;
+#pragma unroll
+            for (int k = 0; k < kEdgeRec; k++)
+                if (ro[k] >= 0) tr[e + 32 * k] = cf[ro[k]];
             if (rank == 0)
-                for (int q = e; q < 2 * g.nrec; q += 32)
-                    trace[(size_t)m * g.nrec * 2 + q] = cf[node_off(a.rec[q >> 1], q & 1, sq)];
+                for (int q = e + 32 * kEdgeRec; q < 2 * g.nrec; q += 32)
+                    tr[q] = cf[node_off(a.rec[q >> 1], q & 1, sq)];
             // side columns 0 and nx-1 (first-order absorbing, from the inward neighbour;
             // they take precedence at the surface and bottom corners)
-            const int oL = node_off(0, 0, sq), oL1 = node_off(1, 0, sq);
-            const int oR = node_off(g.nx - 1, 0, sq), oR1 = node_off(g.nx - 2, 0, sq);
             for (int l = e; l < nrows; l += 32) {
                 const float2 cpcs = coef[l].c;
                 const float *cr = cf + (size_t)l * RS * 2;
@@ -265,7 +296,24 @@ __global__ void __maxnreg__(HOM && !ONE ? kResRegsHom : kResRegs) k_resident(Res
                 nr[oR] = absorb(cr[oR], cr[oR1], cpcs.x);
                 nr[oR + 1] = absorb(cr[oR + 1], cr[oR1 + 1], cpcs.y);
             }
+            // source term: u^{m+1} += dt^2/nu f^m on the patch nodes of this CTA, added last
+            // as in the node update of the streaming kernel
+            if (npw > 0) {
+                asm volatile("bar.sync 1, %0;" :: "r"(32 * (npw + 1)) : "memory");
+#pragma unroll
+                for (int k = 0; k < kNodes; k++)
+                    if (po[k] >= 0) {
+                        nf[po[k]] = add_force(nf[po[k]], S, wx[k]);
+                        nf[po[k] + 1] = add_force(nf[po[k] + 1], S, wz[k]);
+                    }
+            }
+            S = Sn;
+            step_barrier<ONE>();
         }
+    }
+    for (int m = edge ? g.nsteps : 0; m < g.nsteps; m++) {   // the march warps
+        // this thread's even slot in its segment's first row
+        const unsigned cur = slot0 + ((m & 1) ? lvl16 : 0u), nxt = slot0 + ((m & 1) ? 0u : lvl16);
         if (active && l0 < l1) {
             Row2P rn, rc, rs;
             int l = l0;
@@ -390,26 +438,7 @@ __global__ void __maxnreg__(HOM && !ONE ? kResRegsHom : kResRegs) k_resident(Res
         }
         if (patch_warp)
             asm volatile("bar.arrive 1, %0;" :: "r"(32 * (npw + 1)) : "memory");
-        if (edge && npw > 0) {
-            // source term: u^{m+1} += dt^2/nu f^m on the patch nodes of this CTA, added last
-            // as in the node update of the streaming kernel (one node per lane)
-            asm volatile("bar.sync 1, %0;" :: "r"(32 * (npw + 1)) : "memory");
-            float *nf = reinterpret_cast<float *>((m & 1) ? A : B);
-            const float S = stf[m];
-            for (int k = tid - a.nmarch; k < kPatch * kPatch; k += 32) {
-                const int bb = k / kPatch, ai = k - bb * kPatch;
-                const int j = sj + bb;
-                if (j < srow0 || j >= srow1) continue;
-                float *row = nf + (size_t)(j - j0) * RS * 2;
-                const int o = node_off(si0 + ai, 0, sq);
-                row[o] = add_force(row[o], S, sw[k]);
-                row[o + 1] = add_force(row[o + 1], S, sw[kPatch * kPatch + k]);
-            }
-        }
-        if (ONE)
-            __syncthreads();
-        else
-            cluster_barrier();
+        step_barrier<ONE>();
     }
     if (rank == 0) {
         const float *row0 = reinterpret_cast<const float *>((g.nsteps & 1) ? B : A);
@@ -443,8 +472,7 @@ static ResShape resident_shape(const Geometry &g, int C, int kmax = 1)
     const int R = (g.nz + C - 1) / C;
     if ((C - 1) * R >= g.nz) return r;   // a CTA would own no rows
     const int sq = npair + 2;   // ghost slots on both sides
-    const size_t smem = (size_t)2 * R * sq * sizeof(float4) + (size_t)R * sizeof(KP) +
-                        2 * kPatch * kPatch * sizeof(float);
+    const size_t smem = (size_t)2 * R * sq * sizeof(float4) + (size_t)R * sizeof(KP);
     if (smem > 227 * 1024) return r;
     int nseg = 1;
     double best = 0.0;
