@@ -237,20 +237,24 @@ __global__ void __maxnreg__(kResRegs) k_resident(ResArgs a)
     const int lfirst = HOM ? (j0 == 0 ? 1 : 0) : l0 + (top ? 1 : 0), llast = min(l1, nrows - 1);
     __syncthreads();
     const KP K0 = coef[min(lfirst, nrows - 1)];
-    bool unif = true;
-    if (!HOM) {
-        bool same = true;
-        if (active)
-            for (int k = lfirst + 1; k < llast; k++) same &= kp_equal(coef[k], K0);
-        unif = __all_sync(0xffffffffu, same) != 0;
-    }
+    // Elsewhere bit k says that the k-th march row has other coefficients than the one before
+    // (from row 31 on, where the shifted-in sign says so, every row reloads): the warps at a layer
+    // interface, which the others wait for, loaded four 16-byte words a row (401x201, three
+    // layers: 618 -> 637 Gcell-upd/s; 101x76, two: 634 -> 667).
+    int change = 0;
+    if (!HOM && active)
+        for (int k = lfirst + 1; k < llast; k++)
+            if (!kp_equal(coef[k], coef[k - 1])) change |= k - lfirst < 31 ? 1 << (k - lfirst) : -1;
+    const bool unif = HOM || __all_sync(0xffffffffu, change == 0) != 0;
     const int npw = __syncthreads_count(patch_warp && (tid & 31) == 0);
     if (!ONE) cluster_barrier();
 
     if (edge) {
         // What the edge warp needs of a step beside u^m it holds in registers: on the step's
         // critical path (the source term comes last, behind the march warps that own the patch)
-        // stand one wait, one shared load, one fma and one store.
+        // stand one wait, one shared load, one fma and one store.  (With the time function, the
+        // receivers' columns and the weights read in the step: one solve of 81x41 in seven CTAs
+        // 0.419 ms for 400 steps against 0.309; 2048 solves 655 Gcell-upd/s against 708.)
         const int e = tid - a.nmarch;
         int ro[kEdgeRec];
 #pragma unroll
@@ -366,6 +370,8 @@ __global__ void __maxnreg__(kResRegs) k_resident(ResArgs a)
                 // pf: a row below the south row exists, prefetch it (every row but the last)
                 // unifK: each lane's march rows share its K0 (no coefficient loads)
                 auto march = [&](auto unifK) {
+                    KP K = K0;
+                    int cg = change;
                     auto row = [&](auto pf, const Row2P &wn, Row2P &wc, Row2P &ws) {
                         row_fromP(pw, pm, px, ws);
                         float4 u = pu;
@@ -378,7 +384,10 @@ __global__ void __maxnreg__(kResRegs) k_resident(ResArgs a)
                             fetch();
                         }
                         southP(wc, ws);
-                        const KP K = decltype(unifK)::value ? K0 : *cf;
+                        if constexpr (!decltype(unifK)::value) {
+                            if (cg & 1) K = *cf;
+                            cg >>= 1;
+                        }
                         pair_updateP(K, wn, wc, ws, u);
                         sts2(se, make_float2(u.x, u.y));
                         sts2(so, make_float2(u.z, u.w));
