@@ -4,10 +4,10 @@
 //
 // CTA r of a cluster of C owns rows [r R, min((r+1) R, nz)) of the grid, both
 // components and both time levels, in its shared memory:
-//     A, B : [R][npair + 2] float4,   coef : [R] KP (FacCoef in (x, z) pairs)
+//     A, B : [R][rs] float2,   coef : [R] KP (FacCoef in (x, z) pairs)
 // A row stores the even columns' (x, z) in sq = npair + 2 float2 slots, then the odd
 // columns' in sq more; slot q of each half belongs to the column pair p = q - 1, and
-// slots 0 and npair + 1 (columns -2, -1, nx.., and column nx when nx is odd) are zero
+// slots 0 and npair + 1 (columns -2, -1, nx..) are zero
 // ghosts.  A thread owning pair p reads its whole neighbourhood, both components at
 // once, with four 64-bit loads (its two columns, the west column from the odd half
 // and the east column from the even half), each at an 8-byte stride across the
@@ -32,7 +32,9 @@
 // them (named barrier 1).  The arithmetic runs on packed
 // (x, z) pairs (.f32x2).  HBM traffic is only the seismogram samples and the source
 // time function: the wavefield never leaves the chip, so this kernel is bound by
-// shared-memory latency and throughput and the per-step barrier, not by HBM.
+// the shared-memory pipe and the per-step barrier, not by HBM: eight 64-bit accesses per
+// column pair, row and step keep the pipe 87% busy on 81x41 (three CTAs an SM, 766 Gcell-upd/s),
+// 79% on 101x76 (695) and 66% on 401x201 (clusters of six, 696; 138 of 152 SMs have a CTA).
 #include <type_traits>
 
 #include "pair_math.cuh"
@@ -47,6 +49,7 @@ namespace oed {
 constexpr int kResThreads = 640;
 constexpr int kResRegs = 96;
 constexpr int kEdgeRec = 6;   // receiver offsets a lane of the edge warp keeps (96 receivers)
+constexpr int kEdgeRows = 2;  // rows of the slab whose absorbing speeds a lane of it keeps
 constexpr size_t kSmemPerSm = 228 * 1024;   // shared memory of an SM, 1 KB of it reserved per CTA
 
 struct ResArgs {
@@ -57,10 +60,12 @@ struct ResArgs {
     const int *rec;                // [nrec]
     Geometry g;
     int R;                         // rows per CTA
-    int sq;                        // float2 slots per half row (npair + 2); a row is 2 sq
+    int sq;                        // float2 slots per half row, npair + 2
+    int rs;                        // float2 slots per row, 2 sq and the padding
     int npair;                     // column pairs per row, (nx + 1) / 2
+    int np;                        // threads per segment, npair and the idle ones
     int nseg;                      // row segments per column pair
-    int rps;                       // rows per segment
+    int rps;                       // rows per segment (the last takes what is left)
     int nmarch;                    // threads of the march warps; the last warp is the edge warp
 };
 
@@ -133,9 +138,10 @@ __device__ __forceinline__ float4 pair_at(unsigned a, unsigned so8)
 
 // The pair's slots in the level being written (u^{m-1} in, u^{m+1} out), at per-thread
 // byte offsets offE (column c) and offO (column c + 1) from a: 0 and so8 for interior pairs.  A
-// side column (or the ghost column nx) is written by the edge warp, not by the march, so
-// its thread's slot is moved to a ghost slot that no thread reads (even slot 0, or slot
-// npair + 1 of either half): the march's stores stay unconditional.
+// side column is written by the edge warp, not by the march, so its thread's slot is moved to a
+// ghost slot that no thread reads (even slot 0, or slot npair + 1 of either half): the march's
+// stores stay unconditional.  (The ghost column nx of an odd width is read by the thread of the
+// side column nx - 1 alone, whose results are not used.)
 __device__ __forceinline__ float4 pair_at_n(unsigned a, int offE, int offO)
 {
     const float2 e = lds2(a + offE), o = lds2(a + offO);
@@ -169,11 +175,9 @@ __device__ __forceinline__ void load_row_remote(unsigned a, unsigned so8, unsign
     row_fromP(ld_cluster2(b + so8 - 8u), make_float4(e.x, e.y, o.x, o.y), ld_cluster2(b + 8u), r);
 }
 
-// float offset of node (column i, component comp) within a shared row
-__device__ __forceinline__ int node_off(int i, int comp, int sq)
-{
-    return 2 * ((i & 1) ? sq + (i >> 1) + 1 : (i >> 1) + 1) + comp;
-}
+// slot of column i within a shared row, and the float offset of its component comp
+__device__ __forceinline__ int node_slot(int i, int sq) { return (i & 1) ? sq + (i >> 1) + 1 : (i >> 1) + 1; }
+__device__ __forceinline__ int node_off(int i, int comp, int sq) { return 2 * node_slot(i, sq) + comp; }
 
 // HOM: the medium is homogeneous, so every march row has the coefficients of row 1.
 // ONE: clusters of one CTA, no remote rows and a CTA barrier in place of the cluster's.
@@ -187,15 +191,14 @@ __global__ void __maxnreg__(kResRegs) k_resident(ResArgs a)
     const int R = a.R, sq = a.sq;
     const int j0 = (int)rank * R;
     const int nrows = max(0, min(R, g.nz - j0));
-    const int lvl = R * sq;   // 16-byte units per level
-    const int RS = 2 * sq;    // float2 slots per row
+    const int RS = a.rs;
     float2 *A = reinterpret_cast<float2 *>(smem4), *B = A + R * RS;
-    KP *coef = reinterpret_cast<KP *>(smem4 + 2 * lvl);
-    const unsigned level0 = smem_addr(A), lvl16 = 16u * (unsigned)lvl;   // shared address of level A; B is lvl16 on
+    KP *coef = reinterpret_cast<KP *>(smem4 + R * RS);
+    const unsigned level0 = smem_addr(A), lvl8 = 8u * (unsigned)(R * RS);   // shared address of level A; B is lvl8 on
     const int tid = threadIdx.x;
     const int nthr = blockDim.x;
 
-    for (int k = tid; k < 2 * lvl; k += nthr) smem4[k] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    for (int k = tid; k < R * RS; k += nthr) smem4[k] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     for (int k = tid; k < nrows; k += nthr) coef[k] = pack_coef(a.fac[j0 + k]);
 
     // march threads are packed densely over (segment, pair): a warp may straddle two
@@ -204,17 +207,17 @@ __global__ void __maxnreg__(kResRegs) k_resident(ResArgs a)
     // this needs no synchronisation with the march, and no march warp is slowed down by
     // the absorbing patch of a side column.
     const bool edge = tid >= a.nmarch;
-    const int p = tid % a.npair;
+    const int p = tid % a.np;
     const int c = 2 * p;
-    const int seg = tid / a.npair;
-    const bool active = !edge && seg < a.nseg;
+    const int seg = tid / a.np;
+    const bool active = !edge && seg < a.nseg && p < a.npair;
     const int kind = (c == 0 ? 1 : 0) | (c + 1 == g.nx - 1 ? 2 : 0) | (c == g.nx - 1 ? 4 : 0);
     const unsigned so8 = 8u * (unsigned)sq, rs8 = 8u * (unsigned)RS;   // bytes: half row, row
     const int offE = (kind & 1) ? -8 : ((kind & 4) ? 8 : 0);
-    const int offO = (int)so8 + ((kind & 6) ? 8 : 0);
+    const int offO = (int)so8 + ((kind & 2) ? 8 : 0);
     const int l0 = seg * a.rps;
     const unsigned slot0 = level0 + 8u * (unsigned)(l0 * RS + p + 1);
-    const int l1 = min(l0 + a.rps, nrows);
+    const int l1 = seg == a.nseg - 1 ? nrows : min(l0 + a.rps, nrows);
     const bool top = (j0 + l0 == 0);
     const SourceDesc<float> *sd = a.src + s;
     const int sj = sd->j0, si0 = sd->i0;
@@ -275,8 +278,12 @@ __global__ void __maxnreg__(kResRegs) k_resident(ResArgs a)
                 wz[k] = sd->wz[q];
             }
         }
-        const int oL = node_off(0, 0, sq), oL1 = node_off(1, 0, sq);
-        const int oR = node_off(g.nx - 1, 0, sq), oR1 = node_off(g.nx - 2, 0, sq);
+        const int oL = node_slot(0, sq), oL1 = node_slot(1, sq);
+        const int oR = node_slot(g.nx - 1, sq), oR1 = node_slot(g.nx - 2, sq);
+        float2 sc[kEdgeRows];   // absorbing speeds of the lane's rows
+#pragma unroll
+        for (int k = 0; k < kEdgeRows; k++)
+            sc[k] = e + 32 * k < nrows ? coef[e + 32 * k].c : make_float2(0.0f, 0.0f);
         float S = stf[0];
         for (int m = 0; m < g.nsteps; m++) {
             const float *cf = reinterpret_cast<const float *>((m & 1) ? B : A);   // u^m
@@ -291,15 +298,17 @@ __global__ void __maxnreg__(kResRegs) k_resident(ResArgs a)
                     tr[q] = cf[node_off(a.rec[q >> 1], q & 1, sq)];
             // side columns 0 and nx-1 (first-order absorbing, from the inward neighbour;
             // they take precedence at the surface and bottom corners)
-            for (int l = e; l < nrows; l += 32) {
-                const float2 cpcs = coef[l].c;
-                const float *cr = cf + (size_t)l * RS * 2;
-                float *nr = nf + (size_t)l * RS * 2;
-                nr[oL] = absorb(cr[oL], cr[oL1], cpcs.x);
-                nr[oL + 1] = absorb(cr[oL + 1], cr[oL1 + 1], cpcs.y);
-                nr[oR] = absorb(cr[oR], cr[oR1], cpcs.x);
-                nr[oR + 1] = absorb(cr[oR + 1], cr[oR1 + 1], cpcs.y);
-            }
+            auto side = [&](int l, float2 k) {
+                const float2 *cr = reinterpret_cast<const float2 *>(cf) + l * RS;
+                float2 *nr = reinterpret_cast<float2 *>(nf) + l * RS;
+                const float2 L = cr[oL], L1 = cr[oL1], Q = cr[oR], Q1 = cr[oR1];
+                nr[oL] = make_float2(absorb(L.x, L1.x, k.x), absorb(L.y, L1.y, k.y));
+                nr[oR] = make_float2(absorb(Q.x, Q1.x, k.x), absorb(Q.y, Q1.y, k.y));
+            };
+#pragma unroll
+            for (int k = 0; k < kEdgeRows; k++)
+                if (e + 32 * k < nrows) side(e + 32 * k, sc[k]);
+            for (int l = e + 32 * kEdgeRows; l < nrows; l += 32) side(l, coef[l].c);
             // source term: u^{m+1} += dt^2/nu f^m on the patch nodes of this CTA, added last
             // as in the node update of the streaming kernel
             if (npw > 0) {
@@ -317,7 +326,7 @@ __global__ void __maxnreg__(kResRegs) k_resident(ResArgs a)
     }
     for (int m = edge ? g.nsteps : 0; m < g.nsteps; m++) {   // the march warps
         // this thread's even slot in its segment's first row
-        const unsigned cur = slot0 + ((m & 1) ? lvl16 : 0u), nxt = slot0 + ((m & 1) ? 0u : lvl16);
+        const unsigned cur = slot0 + ((m & 1) ? lvl8 : 0u), nxt = slot0 + ((m & 1) ? 0u : lvl8);
         if (active && l0 < l1) {
             Row2P rn, rc, rs;
             int l = l0;
@@ -459,7 +468,7 @@ __global__ void __maxnreg__(kResRegs) k_resident(ResArgs a)
 // Shape of the resident launch for a grid: cluster size C (1..8) and rows per CTA,
 // or C = 0 when the two levels do not fit in C CTAs of shared memory.
 struct ResShape {
-    int C, R, sq, npair, nseg, rps, nmarch, threads;
+    int C, R, sq, rs, npair, np, nseg, rps, nmarch, threads;
     size_t smem;
 };
 
@@ -481,11 +490,11 @@ static ResShape resident_shape(const Geometry &g, int C, int kmax = 1)
     const int R = (g.nz + C - 1) / C;
     if ((C - 1) * R >= g.nz) return r;   // a CTA would own no rows
     const int sq = npair + 2;   // ghost slots on both sides
-    const size_t smem = (size_t)2 * R * sq * sizeof(float4) + (size_t)R * sizeof(KP);
-    if (smem > 227 * 1024) return r;
-    int nseg = 1;
+    auto bytes = [&](int rs) { return (size_t)R * rs * sizeof(float4) + (size_t)R * sizeof(KP); };
+    if (bytes(2 * sq) > 227 * 1024) return r;
+    int nseg = 1, per_sm = 1;
     double best = 0.0;
-    for (int k = 1; k <= kmax && k <= 10 && k * (smem + 1024) <= kSmemPerSm; k++) {
+    for (int k = 1; k <= kmax && k <= 10 && k * (bytes(2 * sq) + 1024) <= kSmemPerSm; k++) {
         const int warps = kResThreads / 32 / k;   // of one CTA; the last one is the edge warp
         const int most = (warps - 1) * 32 / npair;
         if (most < 1) break;
@@ -495,17 +504,39 @@ static ResShape resident_shape(const Geometry &g, int C, int kmax = 1)
         if (score > best) {
             best = score;
             nseg = n;
+            per_sm = k;
         }
     }
+    // A warp that straddles two segments reads two runs of slots: without bank conflicts if a
+    // segment's first slot lies as many slots behind the one before, modulo the 16 slots of a
+    // 64-bit access, as its first thread lies threads behind.  Rows get up to 15 slots of padding
+    // for that, segments an idle thread or a row less (the last has it then), as far as the plan's
+    // warps and CTAs per SM allow.  Gcell-upd/s without and with: 61x31 672 and 774, 81x41 712
+    // and 766, 121x61 606 and 663, 151x76 712 and 777, 201x101 662 and 711, 401x201 684 and 696
+    // (the side columns' 64-bit accesses included).
+    r.rs = 2 * sq;
+    r.np = npair;
+    r.rps = (R + nseg - 1) / nseg;
+    const int rows = r.rps, threads = (npair * nseg + 31) / 32 * 32;
+    bool found = nseg == 1;
+    for (int np = npair; np < npair + 16 && np * nseg <= threads && !found; np++)
+        for (int rps = rows; rps > 0 && R - (nseg - 1) * rps <= rows && !found; rps--)
+            for (int rs = 2 * sq; rs < 2 * sq + 16 && !found; rs++) {
+                if ((rps * rs - np) % 16 || R - (nseg - 1) * rps < 1) continue;
+                if (bytes(rs) > 227 * 1024 || per_sm * (bytes(rs) + 1024) > kSmemPerSm) continue;
+                found = true;
+                r.rs = rs;
+                r.np = np;
+                r.rps = rps;
+            }
     r.C = C;
     r.R = R;
     r.sq = sq;
     r.npair = npair;
     r.nseg = nseg;
-    r.rps = (R + nseg - 1) / nseg;
-    r.nmarch = (npair * nseg + 31) / 32 * 32;
+    r.nmarch = threads;
     r.threads = r.nmarch + 32;
-    r.smem = smem;
+    r.smem = bytes(r.rs);
     return r;
 }
 
@@ -594,6 +625,8 @@ cudaError_t launch_resident(const oed_ctx *ctx, int C, int nsolve, cudaStream_t 
     if (nsteps_override > 0 && nsteps_override < a.g.nsteps) a.g.nsteps = nsteps_override;
     a.R = r.R;
     a.sq = r.sq;
+    a.rs = r.rs;
+    a.np = r.np;
     a.npair = r.npair;
     a.nseg = r.nseg;
     a.rps = r.rps;
