@@ -31,10 +31,13 @@
 // the source term to the patch nodes once the march warps that own them have stored
 // them (named barrier 1).  The arithmetic runs on packed
 // (x, z) pairs (.f32x2).  HBM traffic is only the seismogram samples and the source
-// time function: the wavefield never leaves the chip, so this kernel is bound by
-// the shared-memory pipe and the per-step barrier, not by HBM: eight 64-bit accesses per
-// column pair, row and step keep the pipe 87% busy on 81x41 (three CTAs an SM, 766 Gcell-upd/s),
-// 79% on 101x76 (695) and 66% on 401x201 (clusters of six, 696; 138 of 152 SMs have a CTA).
+// time function: the wavefield never leaves the chip, so this kernel is bound by the
+// shared-memory pipe (eight 64-bit accesses per column pair, row and step) and the per-step
+// barrier, not by HBM.  Large launches: 81x41 867 Gcell-upd/s (three CTAs an SM), 101x76, two
+// layers, 722, 151x76, three layers, 784, 201x101 706, 401x201 692 (clusters of six: 138 of 152 SMs
+// have a CTA).
+#include <algorithm>
+#include <cmath>
 #include <type_traits>
 
 #include "pair_math.cuh"
@@ -43,9 +46,7 @@ namespace oed {
 
 // Block size and register cap: registers are split over the SM's four schedulers
 // (16 K each), so 20 warps of 96 registers is the most one CTA can hold (the packed
-// update needs about 90).  The last warp is the edge warp; three row segments of about
-// twelve rows per column pair (19 march warps at 401 columns) measured faster than one,
-// two, four or five.
+// update needs about 90).  The last warp is the edge warp.
 constexpr int kResThreads = 640;
 constexpr int kResRegs = 96;
 constexpr int kEdgeRec = 6;   // receiver offsets a lane of the edge warp keeps (96 receivers)
@@ -64,6 +65,7 @@ struct ResArgs {
     int rs;                        // float2 slots per row, 2 sq and the padding
     int npair;                     // column pairs per row, (nx + 1) / 2
     int np;                        // threads per segment, npair and the idle ones
+    int shift;                     // 1: segments start below the surface row
     int nseg;                      // row segments per column pair
     int rps;                       // rows per segment (the last takes what is left)
     int nmarch;                    // threads of the march warps; the last warp is the edge warp
@@ -215,10 +217,15 @@ __global__ void __maxnreg__(kResRegs) k_resident(ResArgs a)
     const unsigned so8 = 8u * (unsigned)sq, rs8 = 8u * (unsigned)RS;   // bytes: half row, row
     const int offE = (kind & 1) ? -8 : ((kind & 4) ? 8 : 0);
     const int offO = (int)so8 + ((kind & 2) ? 8 : 0);
-    const int l0 = seg * a.rps;
+    // The rows are cut into segments of rps rows.  The surface row, and the slab's last row, are no
+    // march rows; the segments that hold them take them besides.  With shift the surface row is not
+    // counted, so that the lanes of a warp that straddles segments run the same loop.
+    const bool top = rank == 0 && seg == 0;
+    const int shift = ONE ? 1 : (rank == 0 ? a.shift : 0);
+    const int l0 = seg * a.rps + (top ? 1 : shift);     // first march row
+    const int l1 = seg == a.nseg - 1 ? nrows : min((seg + 1) * a.rps + shift, nrows);
+    const bool rows = active && (top || l0 < l1);
     const unsigned slot0 = level0 + 8u * (unsigned)(l0 * RS + p + 1);
-    const int l1 = seg == a.nseg - 1 ? nrows : min(l0 + a.rps, nrows);
-    const bool top = (j0 + l0 == 0);
     const SourceDesc<float> *sd = a.src + s;
     const int sj = sd->j0, si0 = sd->i0;
     const int siA = c - sd->i0, siB = c + 1 - sd->i0;
@@ -230,14 +237,14 @@ __global__ void __maxnreg__(kResRegs) k_resident(ResArgs a)
     // barrier 1 after their march (without waiting), the edge warp waits there.  The
     // count is fixed per CTA, so every step's barrier completes.
     const int srow0 = max(sj, j0), srow1 = min(sj + kPatch, j0 + nrows);   // patch rows in this CTA
-    const bool patch = active && (scolA || scolB) && sj + kPatch > j0 + l0 && sj < j0 + l1;
+    const bool patch = rows && (scolA || scolB) && sj + kPatch > j0 + (top ? 0 : l0) && sj < j0 + l1;
     const bool patch_warp = __any_sync(0xffffffffu, patch);
     float *trace = a.trace + (size_t)s * g.nlev * g.nrec * 2;
     // The march keeps its rows' coefficients in registers instead of reloading them row by
     // row: in a homogeneous medium they are the CTA's, otherwise where the march rows of every
     // lane of a warp (its segment's, without the surface row and the slab's last row, which are
     // peeled) have one set each, as anywhere but around a layer interface.
-    const int lfirst = HOM ? (j0 == 0 ? 1 : 0) : l0 + (top ? 1 : 0), llast = min(l1, nrows - 1);
+    const int lfirst = HOM ? (rank == 0 ? 1 : 0) : l0, llast = min(l1, nrows - 1);
     __syncthreads();
     const KP K0 = coef[min(lfirst, nrows - 1)];
     // Elsewhere bit k says that the k-th march row has other coefficients than the one before
@@ -327,34 +334,25 @@ __global__ void __maxnreg__(kResRegs) k_resident(ResArgs a)
     for (int m = edge ? g.nsteps : 0; m < g.nsteps; m++) {   // the march warps
         // this thread's even slot in its segment's first row
         const unsigned cur = slot0 + ((m & 1) ? lvl8 : 0u), nxt = slot0 + ((m & 1) ? 0u : lvl8);
-        if (active && l0 < l1) {
-            Row2P rn, rc, rs;
+        if (rows) {
+            Row2P rn, rc, rs;   // the rows l - 1 and l
             int l = l0;
-            load_row(cur, so8, rc);
-            unsigned cl = cur, nl = nxt;   // the even slot in row l of u^m, of u^{m+1}
+            if (ONE || l > 0)
+                load_row(cur - rs8, so8, rn);
+            else
+                load_row_remote(cur + (R - 1) * rs8, so8, rank - 1, rn);
+            if (ONE || l < nrows)
+                load_row(cur, so8, rc);
+            else   // a one-row slab below the surface
+                load_row_remote(cur - rs8, so8, rank + 1, rc);
+            southP(rn, rc);
             if (top) {   // surface row: no north differences, cross terms on the row itself
-                if (ONE || l + 1 < nrows)
-                    load_row(cur + rs8, so8, rs);
-                else   // a one-row slab
-                    load_row_remote(cur, so8, rank + 1, rs);
-                southP(rc, rs);
-                Row2P nt = rc;
+                Row2P nt = rn;
                 nt.va = nt.vb = make_float2(0.0f, 0.0f);
-                float4 u = pair_at_n(nxt, offE, offO);
-                const KP K = coef[l];
-                pair_updateP(K, nt, rc, rs, u);
-                pair_put_n(nxt, offE, offO, u);
-                rn = rc;
-                rc = rs;
-                l++;
-                cl += rs8;
-                nl += rs8;
-            } else {
-                if (ONE || l > 0)
-                    load_row(cur - rs8, so8, rn);
-                else
-                    load_row_remote(cur + (R - 1) * rs8, so8, rank - 1, rn);
-                southP(rn, rc);
+                float4 u = pair_at_n(nxt - rs8, offE, offO);
+                const KP K = coef[0];
+                pair_updateP(K, nt, rn, rc, u);
+                pair_put_n(nxt - rs8, offE, offO, u);
             }
             // rows whose south neighbour is a local row and that are not the bottom row:
             // unrolled by three with the three window rows taking turns
@@ -362,7 +360,7 @@ __global__ void __maxnreg__(kResRegs) k_resident(ResArgs a)
             if (l < lstop) {
                 // Four shared addresses move down with the march: the even and odd slots of the row
                 // to fetch, and of the row whose u^{m-1} is fetched with it and that is stored next
-                unsigned pe = cl + rs8, po = pe + so8, we = nl + offE, wo = nl + offO;
+                unsigned pe = cur + rs8, po = pe + so8, we = nxt + offE, wo = nxt + offO;
                 const KP *cf = coef + l;
                 // the loads of the next row are issued before the update of this one
                 float4 pm, pu;
@@ -468,20 +466,39 @@ __global__ void __maxnreg__(kResRegs) k_resident(ResArgs a)
 // Shape of the resident launch for a grid: cluster size C (1..8) and rows per CTA,
 // or C = 0 when the two levels do not fit in C CTAs of shared memory.
 struct ResShape {
-    int C, R, sq, rs, npair, np, nseg, rps, nmarch, threads;
+    int C, R, sq, rs, shift, npair, np, nseg, rps, nmarch, threads;
     size_t smem;
 };
 
 // kmax: the most CTAs one SM gets of the launch, so the most that are worth planning for.
 //
-// Small slabs leave room for several CTAs on an SM: fewer, longer segments per CTA (a segment
-// of n rows loads n + 2) and independent step barriers, one CTA computing while another
-// waits, against the most march warps one CTA can have.  The choice is by a fit to the rates
-// measured with 2 to 14 segments and 1 to 6 CTAs per SM: an SM's rate grows by 20 units per
-// march warp and 55 per further CTA from 360.  It takes the fastest of k = 1 .. 6 on every
-// grid tried (Gcell-upd/s, k = 1 first): 61x31 257 -> 620 (k = 6), 81x41 382 -> 658 (3), 101x76
-// in clusters of two 328 -> 570 (3), 201x101 in clusters of three 446 -> 540 (2); one CTA on
-// 121x61 (542), 151x76 (636) and everything larger.
+// The slab's rows go to nseg segments of rps rows, the last takes what is left.  With no more
+// than one CTA an SM the step's latency counts: the fewest rows a thread.  Otherwise the plan of
+// the highest product of
+//   sqrt(the share of the warps' lanes and rows that hold nodes; the longest segment sets the step),
+//   rows / (rows + 3): what a segment costs besides its rows (the row above it, its start),
+//   warps / (warps + 15): all CTAs' warps on the SM, which hide each other's latency,
+//   balance^(1/6): a CTA's warps go to the SM's four schedulers in turn,
+//   0.92 where straddling warps have bank conflicts, else 0.97 where the edge warp has.
+// A fit to 1050 plans of 29 grids: it takes one 1.9% slower than the best on average.  Against as
+// many segments as a share of the registers' warps allows, scored by warps and CTAs alone,
+// Gcell-upd/s: 41x21 325 -> 551, 50x50 612 -> 717, 64x64 743 -> 803, 81x41 766 -> 867, 101x101 666 ->
+// 722, 101x76 668 -> 722 (two layers), 161x81 in clusters of two 684 -> 738; 401x201 in clusters of six 640 and
+// 643; a few lose: 61x31 774 -> 755, 91x61 777 -> 736, 221x60 826 -> 784, 301x151 656 -> 642.
+//
+// A warp that straddles two segments reads two runs of slots: without bank conflicts if a
+// segment's first slot lies as many slots behind the one before, modulo the 16 slots of a
+// 64-bit access, as its first thread lies threads behind.  Rows get up to 15 slots of padding
+// for that and segments up to 15 idle threads, as far as the warps and the CTAs per SM allow; an
+// odd row also spreads the edge warp's column over the banks.  Gcell-upd/s without and with: 61x31
+// 672 and 774, 81x41 712 and 766, 121x61 606 and 663, 151x76 712 and 777, 201x101 662 and 711,
+// 401x201 684 and 696 (the side columns' 64-bit accesses included).
+//
+// Segments that start below the surface row (shift) have the same number of march rows, so a
+// straddling warp does not diverge (81x41 766 -> 830 Gcell-upd/s, 201x101 in clusters of two 674 -> 701),
+// but the first one takes a row more, and a cluster waits for it: not where straddling warps are
+// few, from four warps a segment on (301x151 in clusters of four 601 and 624, 351x176 in clusters
+// of six 553 and 563).
 static ResShape resident_shape(const Geometry &g, int C, int kmax = 1)
 {
     ResShape r{};
@@ -492,49 +509,46 @@ static ResShape resident_shape(const Geometry &g, int C, int kmax = 1)
     const int sq = npair + 2;   // ghost slots on both sides
     auto bytes = [&](int rs) { return (size_t)R * rs * sizeof(float4) + (size_t)R * sizeof(KP); };
     if (bytes(2 * sq) > 227 * 1024) return r;
-    int nseg = 1, per_sm = 1;
-    double best = 0.0;
-    for (int k = 1; k <= kmax && k <= 10 && k * (bytes(2 * sq) + 1024) <= kSmemPerSm; k++) {
-        const int warps = kResThreads / 32 / k;   // of one CTA; the last one is the edge warp
-        const int most = (warps - 1) * 32 / npair;
-        if (most < 1) break;
-        const int rows = (R + (most < R ? most : R) - 1) / (most < R ? most : R);
-        const int n = (R + rows - 1) / rows;      // segments that have rows
-        const double score = (360.0 + 20.0 * k * ((npair * n + 31) / 32) + 55.0 * (k - 1)) * rows / (rows + 2.0);
-        if (score > best) {
-            best = score;
-            nseg = n;
-            per_sm = k;
-        }
-    }
-    // A warp that straddles two segments reads two runs of slots: without bank conflicts if a
-    // segment's first slot lies as many slots behind the one before, modulo the 16 slots of a
-    // 64-bit access, as its first thread lies threads behind.  Rows get up to 15 slots of padding
-    // for that, segments an idle thread or a row less (the last has it then), as far as the plan's
-    // warps and CTAs per SM allow.  Gcell-upd/s without and with: 61x31 672 and 774, 81x41 712
-    // and 766, 121x61 606 and 663, 151x76 712 and 777, 201x101 662 and 711, 401x201 684 and 696
-    // (the side columns' 64-bit accesses included).
-    r.rs = 2 * sq;
-    r.np = npair;
-    r.rps = (R + nseg - 1) / nseg;
-    const int rows = r.rps, threads = (npair * nseg + 31) / 32 * 32;
-    bool found = nseg == 1;
-    for (int np = npair; np < npair + 16 && np * nseg <= threads && !found; np++)
-        for (int rps = rows; rps > 0 && R - (nseg - 1) * rps <= rows && !found; rps--)
-            for (int rs = 2 * sq; rs < 2 * sq + 16 && !found; rs++) {
-                if ((rps * rs - np) % 16 || R - (nseg - 1) * rps < 1) continue;
-                if (bytes(rs) > 227 * 1024 || per_sm * (bytes(rs) + 1024) > kSmemPerSm) continue;
-                found = true;
+    r.shift = C == 1 || npair < 128;
+    const int top = C == 1, most = std::min((kResThreads - 32) / npair, R);
+    double best = -1.0;
+    for (int n = 1; n <= most; n++)
+        for (int d = -2; d <= 1; d++) {
+            const int rps = (R + n - 1) / n + d, last = R - top - (n - 1) * rps;
+            if (rps < 1 || last < 1 || (n == 1 && d != 0)) continue;
+            const int rows = n == 1 ? R : std::max(rps + top, last);
+            const int warps = (npair * n + 31) / 32;
+            int k = std::min((int)(kSmemPerSm / (bytes(2 * sq) + 1024)), kResThreads / 32 / (warps + 1));
+            k = std::max(1, std::min(k, kmax));
+            int np = npair, rs = 2 * sq;
+            bool found = false;
+            for (int odd = 1; odd >= 0 && !found; odd--)
+                for (int p = npair; p < npair + 16 && p * n <= 32 * warps && !found; p++)
+                    for (int q = 2 * sq + odd; q < 2 * sq + 16 && !found; q += 2)
+                        if ((n == 1 || (rps * q - p) % 16 == 0) && bytes(q) <= 227 * 1024 &&
+                            k * (bytes(q) + 1024) <= kSmemPerSm) {
+                            found = true;
+                            np = p;
+                            rs = q;
+                        }
+            const double full = (double)npair * R / (32.0 * warps * rows);
+            const double sched = warps / (4.0 * ((warps + 3) / 4));
+            const double score = kmax == 1 ? 1.0 / (rows + 0.01 * n)
+                                           : sqrt(full) * rps / (rps + 3.0) * (k * warps) / (k * warps + 15.0) *
+                                                 cbrt(sqrt(sched)) * (found ? (rs & 1 ? 1.0 : 0.97) : 0.92);
+            if (score > best) {
+                best = score;
                 r.rs = rs;
                 r.np = np;
+                r.nseg = n;
                 r.rps = rps;
+                r.nmarch = 32 * warps;
             }
+        }
     r.C = C;
     r.R = R;
     r.sq = sq;
     r.npair = npair;
-    r.nseg = nseg;
-    r.nmarch = threads;
     r.threads = r.nmarch + 32;
     r.smem = bytes(r.rs);
     return r;
@@ -627,6 +641,7 @@ cudaError_t launch_resident(const oed_ctx *ctx, int C, int nsolve, cudaStream_t 
     a.sq = r.sq;
     a.rs = r.rs;
     a.np = r.np;
+    a.shift = r.shift;
     a.npair = r.npair;
     a.nseg = r.nseg;
     a.rps = r.rps;
