@@ -24,11 +24,12 @@
 //
 // What bounds it: HBM, with T = 4 at 8 B per cell-update (801x401, three layers, 672
 // solves: 705 Gcell-upd/s, 83% of the measured copy rate; 70 solves of 1601x801: 730), and
-// with few solves the blocks that do not fill the chip evenly (56 solves: 543; 7 of
-// 1601x801: 519).  The tile kernel it replaces, two steps per pass through shared memory,
+// with few solves the blocks that do not fill the chip evenly (56 solves: 559; 7 of
+// 1601x801: 535).  The tile kernel it replaces, two steps per pass through shared memory,
 // ran these at 362, 340 and 325.  T = 2 (16 B) 390, T = 3 560: two more steps of registers
 // cost less than their bytes.  Eight warps an SM at up to 255 registers: twelve at 168
 // spill (673 on the 672 solves), sixteen much more (360).
+#include <cmath>
 #include <type_traits>
 
 #include "pair_math.cuh"
@@ -388,15 +389,18 @@ static cudaError_t strip_pass(StripArgs a, int nsm, cudaStream_t st)
 {
     constexpr int W = 64 - 2 * ((T + 1) / 2 * 2);
     a.nstrip = (a.g.nx + W - 1) / W;
-    // bands: more of them fill the chip when there are few strips, but each costs about twelve
-    // rows more (2 T rows computed twice, its start).  n warps per SM take the time of n plus
-    // what a round loses while it fills and drains: measured about 3.5 when all are resident
-    // at once, 6.5 when blocks follow one another.
+    // bands: more of them fill the chip when there are few strips, but each costs about 22 rows
+    // more (2 T rows computed twice, its start).  Blocks run in waves of the warps that the chip
+    // holds; the last, partly filled one costs as much as the others.  A fit to 1 to 16 bands on
+    // nine batches (801x401, 1601x801, 701x351, 501x501; 7 to 105 solves): the rule's choice is
+    // 0.2% slower than the best on average.  With a wave's cost spread over its blocks, Gcell-upd/s:
+    // 28 solves of 801x401 443 -> 475, 49 of 701x351 492 -> 513, 56 of 801x401 543 -> 554, 7 of
+    // 1601x801 519 -> 526.
     const double strips = (double)a.nsolve * a.nstrip;
     double best = 0.0;
     for (int nb = 1; nb <= 64 && a.g.nz / nb >= 4 * T; nb++) {
-        const double n = strips * nb / nsm;
-        const double cost = (n + (n > kStripWarps ? 6.5 : 3.5)) * ((double)a.g.nz / nb + 12.0);
+        const double waves = std::ceil(strips * nb / (nsm * kStripWarps));
+        const double cost = waves * ((double)a.g.nz / nb + 22.0);
         if (nb == 1 || cost < best) {
             best = cost;
             a.nband = nb;
