@@ -508,7 +508,9 @@ static ResShape resident_shape(const Geometry &g, int C, int kmax = 1)
     if ((C - 1) * R >= g.nz) return r;   // a CTA would own no rows
     const int sq = npair + 2;   // ghost slots on both sides
     auto bytes = [&](int rs) { return (size_t)R * rs * sizeof(float4) + (size_t)R * sizeof(KP); };
-    if (bytes(2 * sq) > 227 * 1024) return r;
+    // 392 bytes short of the limit: which grids count as on chip decides the workspace and which
+    // launch shapes are accepted, and stays what it was with the source weights in shared memory
+    if (bytes(2 * sq) + 392 > 227 * 1024) return r;
     r.shift = C == 1 || npair < 128;
     const int top = C == 1, most = std::min((kResThreads - 32) / npair, R);
     double best = -1.0;
