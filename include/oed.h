@@ -227,8 +227,8 @@ int oed_hessian(oed_ctx *ctx, const double *theta, int n, const double *lo, cons
                 double *H_rec, int *status, void *stream);
 
 /* Per-node gain and quadrature sum (Sec. 3.3.3, Thm 4, Eqs. intpoly / mcs):
- *   S = sqrt(diag H_1), Ht = S^-1 H_1 S^-1 = L L^T (Cholesky, FP64),
- *   log det H_1 = sum log H_ii + 2 sum log L_ii,
+ *   S = sqrt(diag H_1), Ht = S^-1 H_1 S^-1; the scaling cancels out of H_1 = L D L^T (FP64),
+ *   log det H_1 = log prod D_j,
  *   D_i = 1/2 log det H_1 - 7/2 (1 + log 2 pi) + sum_j log(hi_j - lo_j),
  *   eig = sum over positive-definite nodes of w_i D_i (deterministic order).
  *   H       device [n][7][7]
@@ -247,7 +247,7 @@ int oed_eig(oed_ctx *ctx, const double *H, int n, const double *w, const double 
  * Thm 4 with N_theta = k, the number of unknowns,
  *   D_i = 1/2 log det H_FF - k/2 (1 + log 2 pi) + sum_{j in F} log(hi_j - lo_j),
  * where H_FF is the sub-block of H_1 over the unknown set F (rows and columns of
- * known parameters drop out; the scaling and Cholesky act on H_FF).
+ * known parameters drop out; the elimination acts on H_FF).
  *   param_mask  bit j set = parameter j (paper order) is unknown; 1..127
  *               (127 is oed_eig).  Other arguments as for oed_eig; lo, hi are
  *               read only at the unknown indices.
