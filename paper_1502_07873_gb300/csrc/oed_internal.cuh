@@ -57,7 +57,8 @@ struct __align__(16 * sizeof(real)) RowCoef {
 // on interior rows.  On the surface row the north terms vanish (naxzm = nazzm = 0)
 // and the cross terms use the row itself: dz_n -> dz_c, dx_n -> dx_c, with
 // nqx = mxm - lx, nqz = lzm - mz.  cp, cs as in RowCoef.  Built from the FP64
-// coefficients by the same kernel.
+// coefficients by the same kernel.  pad0 .. pad3 serve the dual problem: the centre
+// coefficients 2 - 2 axx - axzp + naxzm and 2 - 2 azx - azzp + nazzm, and 1 - cp, 1 - cs.
 template <typename real>
 struct __align__(16 * sizeof(real)) FacCoef {
     real axx, axzp, naxzm, px, nqx, azx, azzp, nazzm, pz, nqz, cp, cs, pad0, pad1, pad2, pad3;
