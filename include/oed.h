@@ -317,7 +317,8 @@ int oed_hessian_map(oed_ctx *ctx, double *theta, int n, const double *y, const d
  *   eps      device [N][D]  the noise realisations (the caller draws them)
  *   g_inner  device [M][D]  data of the inner (evidence) samples; passing the
  *                           outer set again gives the sample-reusing variant
- *   log_ev   device [N]; eig device [1] or NULL
+ *   log_ev   device [N]; eig device [1] or NULL.  A distance that is NaN makes its row's
+ *            log_ev NaN; a row with no comparable distance (all NaN or infinite) gets -inf
  * N, M, D >= 1, sigma > 0, else OED_EINVAL.  Asynchronous on `stream`. */
 int oed_dlmc(const double *g_outer, const double *eps, int N, const double *g_inner, int M, int D,
              double sigma, double *log_ev, double *eig, void *stream);

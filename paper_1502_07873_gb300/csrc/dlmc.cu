@@ -131,13 +131,15 @@ __global__ void __launch_bounds__(256) k_screen(const float *__restrict__ val, i
 constexpr int kEvWarps = 4, kEvPer = 8, kEvList = 2048;   // warps, samples a lane looks at per round, list
 constexpr int kEvShared = 12288;   // longest data row kept in shared memory (96 KB)
 
-// (max, sum) of a warp's lanes; every lane gets them
+// (max, sum) of a warp's lanes; every lane gets them.  A lane without a comparable distance holds
+// (-inf, 0), or (-inf, NaN) after a distance that is NaN: its sum goes on as it is, so a NaN meets
+// the samples of the other lanes and warps.
 __device__ __forceinline__ void warp_log_sum(double &mx, double &sm)
 {
     double top = mx;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) top = fmax(top, __shfl_xor_sync(0xffffffffu, top, o));
-    double s = top > -INFINITY ? sm * exp(mx - top) : 0.0;
+    double s = mx > -INFINITY ? sm * exp(mx - top) : sm;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     mx = top;
@@ -264,7 +266,8 @@ __global__ void __launch_bounds__(32 * kEvWarps) k_log_evidence(
         mx = lane < kEvWarps ? red[0][lane] : -INFINITY;
         sm = lane < kEvWarps ? red[1][lane] : 0.0;
         warp_log_sum(mx, sm);
-        if (lane == 0) log_ev[n] = mx + log(sm) - log_m;
+        // (a row without one comparable distance: -inf)
+        if (lane == 0) log_ev[n] = mx > -INFINITY ? mx + log(sm) - log_m : -INFINITY;
     }
 }
 
