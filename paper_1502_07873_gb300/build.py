@@ -19,7 +19,7 @@ SOURCES = ["api.cu", "source.cu", "stencil.cu", "stream_tma.cu", "stream_strip.c
            "noalloc.cu", "smolyak.cpp", "server.cpp"]
 HEADERS = [os.path.join(CSRC, "oed_internal.cuh"), os.path.join(CSRC, "stencil_cell.cuh"),
            os.path.join(CSRC, "nvtx_range.h"), os.path.join(CSRC, "pair_math.cuh"),
-           os.path.join(CSRC, "tma_sync.cuh"),
+           os.path.join(CSRC, "tma_sync.cuh"), os.path.join(CSRC, "dlmc_groups.h"),
            os.path.join(ROOT, "include", "oed.h")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

@@ -28,13 +28,13 @@
 #include <algorithm>
 #include <cmath>
 
+#include "dlmc_groups.h"
 #include "oed_internal.cuh"
 
 namespace oed {
 
-constexpr int kSN = 64, kSM = 64, kSD = 32;      // k_screen: block tile and chunk of the data dimension
+constexpr int kSN = kScreenRows, kSM = 64, kSD = 32;      // k_screen: block tile and chunk of the data dimension
 constexpr int kDropBits = 60;
-constexpr size_t kScreenFloats = (size_t)1 << 25;   // distances held at once (128 MB); rows go in groups
 
 // y_n = g_outer[n] + eps[n], scaled and rounded to FP32; g likewise
 __device__ __forceinline__ float screen_value(double v, double scale) { return (float)(v * scale); }
@@ -310,8 +310,7 @@ extern "C" int oed_dlmc(const double *g_outer, const double *eps, int N, const d
     // scratch: [N] |eps|^2, the screened values, the distances of a group of rows, [N] smallest
     // distances, the largest norm.  Without it (the device is full) every pair is kept, at more time.
     const int Dp = (D + kSD - 1) / kSD * kSD;
-    const size_t held = std::min((size_t)N * M, kScreenFloats);
-    const int rows = (int)std::min((size_t)N, std::max(held / M / kSN * kSN, (size_t)kSN));
+    const int rows = dlmc_group_rows(N, M);
     const size_t nval = ((size_t)N + M) * Dp, ndist = (size_t)rows * M;
     double *e2 = nullptr;
     if (cudaMallocAsync((void **)&e2, (size_t)N * 8 + (nval + ndist + N + 1) * 4, st) != cudaSuccess) {
