@@ -46,14 +46,15 @@ __global__ void __launch_bounds__(256) k_screen_values(const double *__restrict_
                                                        int N, const double *__restrict__ g_in, int M, int D, int Dp,
                                                        double scale, float *__restrict__ val, unsigned *__restrict__ gmax)
 {
-    const int r = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (r >= N + M) return;
+    const size_t r = (size_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+    const int lane = threadIdx.x & 31;
+    if (r >= (size_t)N + M) return;
     float s = 0.0f;
     for (int d = lane; d < Dp; d += 32) {
         float v = 0.0f;
-        if (d < D) v = r < N ? screen_value(g_out[(size_t)r * D + d] + eps[(size_t)r * D + d], scale)
-                             : -screen_value(g_in[(size_t)(r - N) * D + d], scale);
-        val[(size_t)r * Dp + d] = v;
+        if (d < D) v = r < N ? screen_value(g_out[r * D + d] + eps[r * D + d], scale)
+                             : -screen_value(g_in[(r - N) * D + d], scale);
+        val[r * Dp + d] = v;
         s = fmaf(v, v, s);
     }
     if (r < N) return;
@@ -161,7 +162,7 @@ __global__ void __launch_bounds__(32 * kEvWarps) k_log_evidence(
     const int n = n0 + blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     float ynorm = 0.0f;
     double e = 0.0;
-    for (int d = tid; d < D; d += blockDim.x) {
+    for (unsigned d = tid; d < (unsigned)D; d += blockDim.x) {
         const double ep = eps[(size_t)n * D + d];
         if (SHARED) ys[d] = g_out[(size_t)n * D + d] + ep;
         e = fma(ep, ep, e);
@@ -198,20 +199,20 @@ __global__ void __launch_bounds__(32 * kEvWarps) k_log_evidence(
     auto data = [&](int d) { return SHARED ? ys[d] : g_out[(size_t)n * D + d] + eps[(size_t)n * D + d]; };
     double mx = -INFINITY, sm = 0.0;
     const float *row = dist ? dist + (size_t)blockIdx.x * M : nullptr;
-    for (int m0 = 0; m0 < M;) {
+    for (unsigned m0 = 0; m0 < (unsigned)M;) {   // (unsigned: a round ends up to 1023 samples past M)
         // the next samples to keep, in order, up to a full list
         int have = 0;
         __syncthreads();
-        while (m0 < M && have + kEvPer * (int)blockDim.x <= kEvList) {
+        while (m0 < (unsigned)M && have + kEvPer * (int)blockDim.x <= kEvList) {
             // a warp takes kEvPer x 32 consecutive samples; kept unless known to be above the
             // limit (NaN and overflow are kept)
             unsigned b[kEvPer];
             int mine = 0;
 #pragma unroll
             for (int q = 0; q < kEvPer; q++) {
-                const int m = m0 + (warp * kEvPer + q) * 32 + lane;
-                const float v = row && m < M ? row[m] : 0.0f;
-                b[q] = __ballot_sync(0xffffffffu, m < M && (!(v > limit) || !(v < 3e38f)));
+                const unsigned m = m0 + (warp * kEvPer + q) * 32 + lane;
+                const float v = row && m < (unsigned)M ? row[m] : 0.0f;
+                b[q] = __ballot_sync(0xffffffffu, m < (unsigned)M && (!(v > limit) || !(v < 3e38f)));
                 mine += __popc(b[q]);
             }
             if (lane == 0) wcount[warp] = mine;
@@ -223,10 +224,10 @@ __global__ void __launch_bounds__(32 * kEvWarps) k_log_evidence(
             }
 #pragma unroll
             for (int q = 0; q < kEvPer; q++) {
-                if (b[q] >> lane & 1) list[at + __popc(b[q] & ((1u << lane) - 1u))] = m0 + (warp * kEvPer + q) * 32 + lane;
+                if (b[q] >> lane & 1) list[at + __popc(b[q] & ((1u << lane) - 1u))] = (int)(m0 + (warp * kEvPer + q) * 32 + lane);
                 at += __popc(b[q]);
             }
-            m0 += kEvPer * (int)blockDim.x;
+            m0 += kEvPer * blockDim.x;
             __syncthreads();
         }
         for (int k = tid; k < have; k += blockDim.x) {
@@ -280,7 +281,7 @@ __global__ void __launch_bounds__(512) k_dlmc_sum(const double *__restrict__ eps
     __shared__ double sv[512];
     const int t = threadIdx.x, T = blockDim.x;
     double v = 0.0;
-    for (int n = t; n < N; n += T) {
+    for (long long n = t; n < N; n += T) {
         double q = 0.0;
         if (e2)
             q = e2[n];
@@ -331,10 +332,9 @@ extern "C" int oed_dlmc(const double *g_outer, const double *eps, int N, const d
     const float slack = (float)((kDropBits * 0.6931471805599453 + log_m) * 1.000001);
     if (shared)
         cudaFuncSetAttribute(k_log_evidence<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kEvShared * 8);
-    for (int n0 = 0; n0 < N; n0 += rows) {
-        const int n1 = std::min(N, n0 + rows);
+    dlmc_for_groups(N, M, [&](int n0, int n1) {
         if (dist)
-            k_screen<<<dim3((M + kSM - 1) / kSM, (n1 - n0 + kSN - 1) / kSN), 256, 0, st>>>(val, N, n0, n1, M, Dp, dist,
+            k_screen<<<dim3((M - 1) / kSM + 1, (n1 - n0 - 1) / kSN + 1), 256, 0, st>>>(val, N, n0, n1, M, Dp, dist,
                                                                                           best);
         if (shared)
             k_log_evidence<true><<<n1 - n0, 32 * kEvWarps, (size_t)D * 8, st>>>(
@@ -342,7 +342,7 @@ extern "C" int oed_dlmc(const double *g_outer, const double *eps, int N, const d
         else
             k_log_evidence<false><<<n1 - n0, 32 * kEvWarps, 0, st>>>(
                 g_outer, eps, n0, g_inner, M, D, Dp, inv2s2, log_m, slack, val, dist, best, gmax, vec, log_ev, e2);
-    }
+    });
     if (eig) k_dlmc_sum<<<1, 512, 0, st>>>(eps, e2, log_ev, N, D, inv2s2, eig);
     if (e2) cudaFreeAsync(e2, st);
     return cudaGetLastError() == cudaSuccess ? OED_OK : OED_ECUDA;

@@ -17,4 +17,13 @@ inline int dlmc_group_rows(int N, int M)
     return (int)std::min((size_t)N, std::clamp(tiles, (size_t)1, (size_t)kScreenTiles) * kScreenRows);
 }
 
+// f(n0, n1) for every group of rows n0 .. n1 - 1 (counted in 64 bits: the end of the last group may
+// lie above the largest int)
+template <typename F>
+inline void dlmc_for_groups(int N, int M, F f)
+{
+    const int rows = dlmc_group_rows(N, M);
+    for (long long n0 = 0; n0 < N; n0 += rows) f((int)n0, (int)std::min((long long)N, n0 + rows));
+}
+
 }  // namespace oed

@@ -34,7 +34,13 @@ int main(int argc, char **argv)
 {
     for (int k = 1; k + 1 < argc; k += 2) {
         const int N = atoi(argv[k]), M = atoi(argv[k + 1]);
-        printf("%d\n", oed::dlmc_group_rows(N, M));
+        long long calls = 0, covered = 0, bad = 0;
+        oed::dlmc_for_groups(N, M, [&](int n0, int n1) {
+            bad += n0 != covered || n1 <= n0 || n1 > N || n1 - n0 > oed::dlmc_group_rows(N, M);
+            covered = n1;
+            if (++calls > 40000000) exit(1);
+        });
+        printf("%d %lld %lld %lld\n", oed::dlmc_group_rows(N, M), calls, covered, bad);
     }
 }
 """
@@ -52,3 +58,8 @@ def test_rows_of_a_group(exe):
         assert (rows + 63) // 64 <= 65535, (n, m, rows)
         assert rows * m <= max(2 ** 25, 64 * m), (n, m, rows)
         assert rows == n or (rows + 64) * m > 2 ** 25 or rows == 65535 * 64, (n, m, rows)   # no smaller than need be
+
+
+def test_groups_cover_the_rows_once(exe):
+    for (n, m), (rows, calls, covered, bad) in zip(SIZES, _run(exe), strict=True):
+        assert bad == 0 and covered == n and calls == -(-n // rows), (n, m, rows, calls, covered, bad)
