@@ -310,8 +310,11 @@ int oed_hessian_map(oed_ctx *ctx, double *theta, int n, const double *y, const d
  * (the Gaussian normalising constant cancels).  Distances are summed in FP64 from
  * the differences (no |y|^2 + |g|^2 - 2 y.g expansion); inner samples whose terms a
  * rigorous FP32 bound puts below 2^-60 of a row's sum, all of them together, are left
- * out.  Scratch is allocated stream-ordered for the call (2^25 floats of distances at
- * most, and the data in FP32); where it does not fit every pair is summed.
+ * out.  Scratch is allocated stream-ordered for the call: the data in FP32 and 2^25
+ * floats of distances at most, or 64 M of them where that is more.  The library keeps
+ * up to 256 MB of it per device for the next call, until a context is destroyed or
+ * oed_create is short of memory.  Where the scratch does not fit every pair is summed,
+ * in another order: the last bits of the results may differ.
  *   g_outer  device [N][D]  noise-free data of the outer samples, e.g. seismograms
  *                           from oed_forward (D = (nsteps+1) * nrec * 2)
  *   eps      device [N][D]  the noise realisations (the caller draws them)

@@ -252,7 +252,12 @@ int oed_create(oed_ctx **out, const oed_problem *p, int max_solves)
 
     const Sizes s = sizes(ctx->g, ctx->precision, max_solves);
     size_t free_b = 0, total_b = 0;
-    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
+    cudaError_t e = cudaMemGetInfo(&free_b, &total_b);
+    if (e == cudaSuccess && s.total > free_b) {
+        scratch_trim();
+        e = cudaMemGetInfo(&free_b, &total_b);
+    }
+    if (e != cudaSuccess) {
         delete ctx;
         return OED_ECUDA;
     }
@@ -263,7 +268,7 @@ int oed_create(oed_ctx **out, const oed_problem *p, int max_solves)
     }
     char *base = nullptr;
     cudaStreamCreateWithFlags(&ctx->own_stream, cudaStreamNonBlocking);
-    cudaError_t e = cudaMallocAsync((void **)&base, s.total, ctx->own_stream);
+    e = cudaMallocAsync((void **)&base, s.total, ctx->own_stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->own_stream);
     if (e != cudaSuccess) {
         cudaStreamDestroy(ctx->own_stream);
@@ -304,6 +309,7 @@ int oed_destroy(oed_ctx *ctx)
     cudaFree(ctx->h_stage_eig);
     cudaFree(ctx->h_stage_bad);
     cudaFree(ctx->d_adj);
+    scratch_trim();
     delete ctx;
     return OED_OK;
 }

@@ -185,6 +185,9 @@ cudaError_t launch_steps_strip(const oed_ctx *ctx, int nsolve, cudaStream_t st, 
                                int nsteps_override);
 void launch_fill_probe(const oed_ctx *ctx, int nsolve, cudaStream_t st);
 
+// dlmc.cu
+void scratch_trim();   // gives back the device memory kept for the double loop's scratch
+
 // resident.cu
 int resident_cluster_size(const oed_ctx *ctx);
 int resident_fits(const Geometry &g);   // smallest cluster holding an FP32 grid, 0 if none
