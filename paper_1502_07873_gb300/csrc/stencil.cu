@@ -158,7 +158,9 @@ __global__ void __launch_bounds__(256) k_step64(StepArgs<double> a, int npair, i
             a.trace[((size_t)s * g.nlev + a.m) * nq + q] = cur[(q & 1) * g.comp_stride + a.rec[q >> 1]];
 
     const int c = 2 * p, last = g.nx - 1;
-    const int j0 = (int)((long long)g.nz * seg / nseg), j1 = (int)((long long)g.nz * (seg + 1) / nseg);
+    // (ZS = 1: one row each, without the divisions)
+    const int j0 = ZS == 1 ? seg : (int)((long long)g.nz * seg / nseg);
+    const int j1 = ZS == 1 ? seg + 1 : (int)((long long)g.nz * (seg + 1) / nseg);
     const bool sideA = c == 0 || c == last, sideB = c + 1 == last, hasB = c + 1 <= last;
     const int iw = c > 0 ? c - 1 : 0, ie = c + 2 <= last ? c + 2 : last;
     // row j of u^m as seen by the pair; outside the grid the neighbour is the node itself
@@ -269,18 +271,24 @@ __global__ void k_gather(const real *__restrict__ cur, real *__restrict__ trace,
         tr[q] = (q & 1 ? cz : cx)[rec[q >> 1]];
 }
 
-// Row segments for the FP64 kernels, columns of which (over all solves) take a thread each:
-// up to zs rows a segment, shorter where that spreads the columns over more of the schedulers
-// (four per SM, each with its own FP64 pipe).  A segment of r rows takes per r + once issue
-// slots, and the warps go round the schedulers.
+// Row segments for the FP64 kernels, columns of which (over all solves) take a thread each: up to zs
+// rows a segment, shorter where that spreads the columns over more of the schedulers (four per SM,
+// each with its own FP64 pipe).  A segment of r rows takes per r + once issue slots of its pipe; the
+// warps go round the pipes, half of a partly filled last round overlaps the others, and a thread's
+// rows follow one another, which a pipe with one or two warps does not hide (latency per row).  A
+// fit to 47 batches of six grids (9x9 to 401x201, 1 to 3000 solves): 1 to 1.5% slower than the best
+// segment length on average.  Counted in whole rounds and without the latency it was 8% and up to
+// 39%: 15 solves of 81x41 482 us for 60 steps against 370 in one-row segments.  These have a kernel
+// without the divisions of the general one (ZS = 1; one solve of 201x101 318 -> 298 us).
 int segments64(long long columns, int nz, int zs, double per, double once)
 {
-    constexpr double kPipes = 4 * 152;
+    constexpr double kPipes = 4 * 152, kLatency = 8.0;
     int best = (nz + zs - 1) / zs;
     double least = 0.0;
     for (int r = zs; r >= 1; r--) {
-        const int nseg = (nz + r - 1) / r;
-        const double cost = std::ceil((double)columns * nseg / 32.0 / kPipes) * (per * ((nz + nseg - 1) / nseg) + once);
+        const int nseg = (nz + r - 1) / r, rows = (nz + nseg - 1) / nseg;
+        const double warps = (double)columns * nseg / 32.0 / kPipes;
+        const double cost = std::max(1.0, 0.5 * (warps + std::ceil(warps))) * (per * rows + once) + kLatency * rows;
         if (r == zs || cost < least) {
             least = cost;
             best = nseg;
@@ -296,7 +304,7 @@ static void launch_one(const oed_ctx *ctx, int nsolve, const StepArgs<real> &a, 
     const Geometry &g = ctx->g;
     const int wz = ctx->tune.wz;
     if constexpr (sizeof(real) == 8) {
-        const int npair = (g.nx + 1) / 2, nseg = segments64((long long)npair * nsolve, g.nz, ZS, 23.0, 12.0);
+        const int npair = (g.nx + 1) / 2, nseg = segments64((long long)npair * nsolve, g.nz, ZS, 23.0, 10.0);
         const long long per = (long long)npair * nseg;
         // 32-bit thread numbers: a batch past them goes in several launches
         const int most = (int)std::max(1LL, std::min((long long)nsolve, (1LL << 31) / per));
@@ -309,7 +317,8 @@ static void launch_one(const oed_ctx *ctx, int nsolve, const StepArgs<real> &a, 
             b.stf += (size_t)s0 * g.nsteps;
             b.trace += (size_t)s0 * g.nlev * g.nrec * 2;
             const unsigned nthr = (unsigned)(per * ns);
-            k_step64<ZS><<<(nthr + 32 * wz - 1) / (32 * wz), 32 * wz, 0, st>>>(b, npair, nseg, nthr);
+            const auto kernel = nseg == g.nz ? k_step64<1> : k_step64<ZS>;
+            kernel<<<(nthr + 32 * wz - 1) / (32 * wz), 32 * wz, 0, st>>>(b, npair, nseg, nthr);
         }
     } else {
         const int rows_per_block = wz * ZS;
