@@ -74,6 +74,8 @@ def kernel_label(t):
         return "cluster-resident, %d CTAs per solve" % t[0]
     if t[0] == -2:
         return "multi-step streaming (four leap-frog steps per pass over column strips, cp.async ring)"
+    if t[0] == -3:
+        return "two-step TMA streaming (two leap-frog steps per pass, persistent, 4-stage mbarrier ring)"
     if t[0] < 0:
         return "TMA streaming (persistent, 4-stage mbarrier ring)"
     return "streaming, %d rows/thread, %d warps/block" % (t[1], t[2])
@@ -162,11 +164,13 @@ def measured_peaks():
 KERNEL_SOURCES = {"k_resident": ("resident.cu", "pair_math.cuh", "stencil_cell.cuh", "oed_internal.cuh"),
                   "k_step": ("stencil.cu", "stencil_cell.cuh", "oed_internal.cuh"),
                   "k_step_tma": ("stream_tma.cu", "tma_sync.cuh", "stencil_cell.cuh", "oed_internal.cuh"),
-                  "k_strip": ("stream_strip.cu", "pair_math.cuh", "stencil_cell.cuh", "oed_internal.cuh")}
+                  "k_strip": ("stream_strip.cu", "pair_math.cuh", "stencil_cell.cuh", "oed_internal.cuh"),
+                  "k_step2_tma": ("stream_tma2.cu", "pair_math.cuh", "tma_sync.cuh", "stencil_cell.cuh",
+                                  "oed_internal.cuh")}
 
 
 def streaming_kernel_name(tuning) -> str:
-    return {-2: "k_strip", -1: "k_step_tma"}.get(tuning[0], "k_step")
+    return {-3: "k_step2_tma", -2: "k_strip", -1: "k_step_tma"}.get(tuning[0], "k_step")
 
 
 def _code_only(text: str) -> str:

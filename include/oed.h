@@ -111,7 +111,7 @@ int oed_destroy(oed_ctx *ctx);
  * for the context's max_solves (oed_workspace_bytes) fits in the context's.  This
  * is how a server keeps one workspace per grid shape resident across requests.
  * Captured time loops are dropped; the kernel choice (oed_autotune /
- * oed_set_tuning), which depends only on the grid shape, is kept.  Streams that
+ * oed_set_tuning), which suits any problem of the grid shape, is kept.  Streams that
  * ran earlier calls on the context must be synchronised first.  Returns OED_OK,
  * OED_EINVAL (malformed problem, another shape or precision, or sensitivity
  * solves with a non-Gaussian time function), OED_ENOMEM (the workspace does not
@@ -139,15 +139,16 @@ int oed_last_step_time(const oed_ctx *ctx, float *ms, int *launches);
  *  - TMA streaming (FP32): the same, with halo tiles moved by the tensor-memory
  *    accelerator into a persistent CTA's mbarrier ring (cluster_size -1);
  *  - multi-step streaming (FP32, grids that do not fit on chip): four steps per
- *    pass over strips of columns (cluster_size -2);
+ *    pass over strips of columns (cluster_size -2), or two per pass over tiles moved
+ *    by the tensor-memory accelerator, faster for one or two solves, media with an
+ *    interface every few rows and wide grids of few rows (cluster_size -3);
  *  - cluster-resident (FP32, grids whose two time levels fit in the shared
  *    memory of a cluster of C <= 8 CTAs, e.g. 401x201): one launch for all
  *    steps, one thread-block cluster per solve, wavefield kept on chip.
  * All give the same node updates, bit for bit.  oed_autotune times every streaming launch
- * shape (rows marched per thread 2/4/8 x warps per block 1/2/4/8), the TMA kernel and
- * every feasible cluster size on nsolve solves of this context's grid, keeps the
- * fastest for later calls, and synchronises the stream; where the multi-step kernel
- * runs it is chosen.  It overwrites the
+ * shape (rows marched per thread 2/4/8 x warps per block 1/2/4/8), the TMA kernel, the
+ * multi-step kernels and every feasible cluster size on nsolve solves of this context's
+ * grid, keeps the fastest for later calls, and synchronises the stream.  It overwrites the
  * context's workspace (no caller data).  nsolve in 1..max_solves, typically
  * 15 * oed_chunk_nodes(ctx). */
 int oed_autotune(oed_ctx *ctx, int nsolve, void *stream);

@@ -419,22 +419,40 @@ int oed_autotune(oed_ctx *ctx, int nsolve, void *stream)
             best = ctx->tune;
         }
     }
-    // multi-step strip kernel (FP32 grids that do not fit on chip).  It is taken whenever it
-    // runs: it moves a third of the one-step kernels' bytes per step (801x401, three layers,
-    // 672 solves: 705 Gcell-upd/s against 247), so the probe only checks that it launches.
-    if (ctx->d_u2 && strip_prepare(ctx) > 0) {
-        ctx->tune = StepTuning{best.zs, best.wz, -2};
+    // multi-step kernels (FP32 grids that do not fit on chip): the strip kernel moves the fewest bytes,
+    // the two-step kernel has the shorter pass and does not mind layer interfaces.  The one-step kernels
+    // are behind both but for a few rows.  us for 100 steps, strip / two-step / one-step:
+    //   801x401, 3 layers: 1 solve 460 / 359 / 424, 3: 511 / 541, 56: 3366 / 5440, 200: 9287 / 18190
+    //   801x401, a layer every 6 rows: 1 solve 656 / 369, 56: 8036 / 5444, 200: 24316 / 18100
+    //   1301x20, 64 solves 906 / 820 / 848; 1217x9, 1 solve 386 / 328 / 310
+    // A probe takes whole passes of both; those under a millisecond are the least of three.
+    if (ctx->d_u2) {
         int probe = std::min(ctx->g.nsteps, std::max(nrep, 16));
-        probe = probe < 4 ? probe : probe / 2 * 2;
-        cudaError_t e = launch_steps_strip(ctx, nsolve, st, e0, e1, 4);   // warm
-        if (e == cudaSuccess) e = launch_steps_strip(ctx, nsolve, st, e0, e1, probe);
-        if (e == cudaSuccess) e = cudaEventSynchronize(e1);
-        float ms = 0.0f;
-        if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
-        if (e != cudaSuccess) return fail(e);
-        ms /= probe;
-        best_ms = ms;
-        best = ctx->tune;
+        if (probe >= 4) probe = probe / 4 * 4;
+        for (int C : {-2, -3}) {
+            if (C == -2 ? strip_prepare(ctx) < 1 : !tma_supported(ctx) || tma2_prepare(ctx) < 1) continue;
+            ctx->tune = StepTuning{best.zs, best.wz, C};
+            const float *last = nullptr;
+            auto launch = [&](int steps) {
+                return C == -2 ? launch_steps_strip(ctx, nsolve, st, e0, e1, steps)
+                               : launch_steps_tma2(ctx, nsolve, st, e0, e1, steps, &last);
+            };
+            cudaError_t e = launch(4);   // warm
+            float ms = 1e30f;
+            for (int k = 0; k < 3 && e == cudaSuccess && (k == 0 || ms < 1.0f); k++) {
+                float one = 0.0f;
+                e = launch(probe);
+                if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+                if (e == cudaSuccess) e = cudaEventElapsedTime(&one, e0, e1);
+                ms = std::min(ms, one);
+            }
+            if (e != cudaSuccess) return fail(e);
+            ms /= probe;
+            if (ms < best_ms) {
+                best_ms = ms;
+                best = ctx->tune;
+            }
+        }
     }
     // cluster-resident kernel (FP32 grids whose two levels fit in 1..8 CTAs)
     const int cmin = resident_cluster_size(ctx);
@@ -509,6 +527,10 @@ int oed_set_tuning(oed_ctx *ctx, int cluster_size, int rows_per_thread, int warp
         if (!ctx->d_u2 || strip_prepare(ctx) < 1)
             return set_err(ctx, OED_EINVAL,
                            "oed_set_tuning: the multi-step kernel needs FP32 and a grid that does not fit on chip");
+    } else if (cluster_size == -3) {
+        if (!ctx->d_u2 || !tma_supported(ctx) || tma2_prepare(ctx) < 1)
+            return set_err(ctx, OED_EINVAL,
+                           "oed_set_tuning: the two-step kernel needs FP32 and a grid that does not fit on chip");
     } else if (cluster_size != 0) {
         const int cmin = resident_cluster_size(ctx);
         if (cmin == 0 || cluster_size < cmin || cluster_size > 8 ||

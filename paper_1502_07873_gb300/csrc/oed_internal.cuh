@@ -89,15 +89,20 @@ struct Geometry {
 // the columns' (x, z) float2 pairs side by side, column c in slot c + 4 of 2 sq slots; the
 // slots of columns -4 .. -1 and past nx - 1 are zero.  A column pair (even c) is 16 bytes
 // on a 16-byte boundary.
+// The paired layout of the two-step kernel takes the same room: sq slots of a row hold the even
+// columns, the next sq the odd ones, column c in slot (c >> 1) + 2 of its half (a half row is a
+// multiple of 16 bytes, a TMA stride).
 __host__ __device__ inline int strip_sq(const Geometry &g) { return ((g.nx + 1) / 2 + 4 + 1) & ~1; }
 __host__ __device__ inline size_t strip_stride(const Geometry &g) { return (size_t)g.nz * 4 * strip_sq(g); }
+__host__ __device__ inline int paired_sq(const Geometry &g) { return strip_sq(g); }
+__host__ __device__ inline size_t paired_stride(const Geometry &g) { return strip_stride(g); }
 
 struct StepTuning {
     int zs;      // streaming kernel: rows marched per thread
     int wz;      // streaming kernel: warps along z in a block
     int C;       // > 0: cluster-resident kernel with clusters of C CTAs (FP32 only);
-                 // -1: TMA streaming kernel (FP32 only); -2: multi-step streaming
-                 // kernel (FP32, grids that do not fit on chip); 0: register streaming kernel
+                 // -1: TMA streaming kernel (FP32 only); -2: multi-step strip kernel, -3: two-step
+                 // TMA kernel (FP32, grids that do not fit on chip); 0: register streaming kernel
 };
 
 }  // namespace oed
@@ -119,9 +124,9 @@ struct oed_ctx {
                                // before every time loop, read when the Hessians are combined)
     void *d_u0 = nullptr;      // wavefield level buffer A [max_solves][2][nz][xp]
     void *d_u1 = nullptr;      // wavefield level buffer B
-    void *d_u2 = nullptr;      // second level pair of the multi-step kernel (FP32 grids
+    void *d_u2 = nullptr;      // second level pair of the multi-step kernels (FP32 grids
     void *d_u3 = nullptr;      // that do not fit on chip; NULL otherwise)
-    void *d_kp = nullptr;      // [nz] the rows' coefficients as (x, z) pairs (multi-step kernel)
+    void *d_kp = nullptr;      // [nz] the rows' coefficients as (x, z) pairs (multi-step kernels)
     void *d_src = nullptr;     // SourceDesc<real>[max_solves]
     void *d_stf = nullptr;     // real [max_solves][nsteps]
     void *d_trace = nullptr;   // real [max_solves][nlev][nrec][2]
@@ -133,6 +138,7 @@ struct oed_ctx {
     int jac_mode = OED_JAC_PAIRS;   // Jacobian form of oed_hessian
     int tma_ctas = 0;               // persistent grid of the TMA streaming kernel
     int strip_sms = 0;              // SMs of the device, set once the multi-step kernel can run
+    int tma2_ctas = 0;              // persistent grid of the two-step TMA kernel
     // host-path staging
     cudaStream_t own_stream = nullptr;
     double *h_stage_theta = nullptr, *h_stage_w = nullptr, *h_stage_H = nullptr,
@@ -168,6 +174,8 @@ void launch_trace_to_f64(const oed_ctx *ctx, int nsolve, double *g, cudaStream_t
 void launch_step_probe(const oed_ctx *ctx, int nsolve, int nrep, cudaStream_t st, cudaEvent_t ev0,
                        cudaEvent_t ev1);
 
+void launch_fill_probe(const oed_ctx *ctx, int nsolve, cudaStream_t st);
+
 int segments64(long long columns, int nz, int zs, double per, double once);   // FP64 row segments
 
 // stream_tma.cu
@@ -183,7 +191,12 @@ int strip_prepare(oed_ctx *ctx);
 void launch_pack_kp(const oed_ctx *ctx, cudaStream_t st);
 cudaError_t launch_steps_strip(const oed_ctx *ctx, int nsolve, cudaStream_t st, cudaEvent_t ev0, cudaEvent_t ev1,
                                int nsteps_override);
-void launch_fill_probe(const oed_ctx *ctx, int nsolve, cudaStream_t st);
+
+// stream_tma2.cu
+int tma2_prepare(oed_ctx *ctx);
+cudaError_t launch_steps_tma2(const oed_ctx *ctx, int nsolve, cudaStream_t st, cudaEvent_t ev0, cudaEvent_t ev1,
+                              int nsteps_override, const float **last);
+void launch_tma2_gather(const oed_ctx *ctx, int nsolve, const float *last, int m, cudaStream_t st);
 
 // dlmc.cu
 void scratch_trim();   // gives back the device memory kept for the double loop's scratch

@@ -96,7 +96,7 @@ struct oed_server {
     std::deque<Request> queue;
     std::map<unsigned long long, Entry> results;
     std::vector<Slot> idle;
-    std::map<std::tuple<int, int, int, int>, std::tuple<int, int, int>> tuning;   // shape, form -> tune
+    std::map<std::tuple<int, int, int, int, int>, std::tuple<int, int, int>> tuning;   // shape, layers, form -> tune
     std::mutex mu;
     std::condition_variable cv_work, cv_done;
     std::vector<std::thread> workers;
@@ -218,7 +218,7 @@ int run_request(oed_server *srv, Request &rq, oed_ctx *ctx, cudaStream_t st, Ent
     int *d_bad = (int *)(d_eig + 1);
     int rc = oed_set_jacobian(ctx, rq.jacobian);
     if (!rc) {
-        const auto key = std::make_tuple(rq.p.nx, rq.p.nz, rq.p.precision, rq.jacobian);
+        const auto key = std::make_tuple(rq.p.nx, rq.p.nz, rq.p.nlayers, rq.p.precision, rq.jacobian);
         std::tuple<int, int, int> tune;
         bool have = false;
         {

@@ -412,8 +412,28 @@ __global__ void k_fill_probe(real *__restrict__ u, size_t n, unsigned salt)
     }
 }
 
+// Source patches without weight, spread over the grid as a batch's are: a multi-step kernel's tiles
+// and strips with a source take longer, and those of a corner are slow without one.
+template <typename real>
+__global__ void k_fill_probe_src(SourceDesc<real> *__restrict__ src, int nsolve, int nx, int nz)
+{
+    const int s = blockIdx.x;
+    SourceDesc<real> &d = src[s];
+    if (threadIdx.x == 0) {
+        const unsigned h = ((unsigned)s + 1u) * 2654435761u;
+        d.i0 = 1 + (int)((h >> 16) % (unsigned)max(1, nx - kPatch - 1));
+        d.j0 = (int)(((h & 0xffffu) * 40503u >> 8) % (unsigned)max(1, nz - kPatch));
+        d.ok = 1;
+    }
+    for (int k = threadIdx.x; k < kPatch * kPatch; k += blockDim.x) d.wx[k] = d.wz[k] = (real)0;
+}
+
 void launch_fill_probe(const oed_ctx *ctx, int nsolve, cudaStream_t st)
 {
+    if (ctx->d_u2) {
+        k_fill_probe_src<float><<<nsolve, 64, 0, st>>>((SourceDesc<float> *)ctx->d_src, nsolve, ctx->g.nx, ctx->g.nz);
+        cudaMemsetAsync(ctx->d_stf, 0, (size_t)nsolve * ctx->g.nsteps * sizeof(float), st);
+    }
     size_t per = ctx->g.solve_stride;
     if (ctx->d_u2) per = per > strip_stride(ctx->g) ? per : strip_stride(ctx->g);
     const size_t n = (size_t)nsolve * per;
@@ -446,6 +466,16 @@ cudaError_t launch_forward_steps(const oed_ctx *ctx, int nsolve, cudaStream_t st
         cudaMemsetAsync(ctx->d_u0, 0, pb, st);
         cudaMemsetAsync(ctx->d_u2, 0, pb, st);
         return launch_steps_strip(ctx, nsolve, st, ev0, ev1, 0);
+    }
+    if (ctx->tune.C == -3) {   // the two-step kernel's paired layout
+        const size_t pb = (size_t)nsolve * paired_stride(ctx->g) * sizeof(float);
+        void *lv[4] = {ctx->d_u0, ctx->d_u1, ctx->d_u2, ctx->d_u3};
+        for (void *p : lv) cudaMemsetAsync(p, 0, pb, st);
+        const float *last = nullptr;
+        const cudaError_t e = launch_steps_tma2(ctx, nsolve, st, ev0, ev1, 0, &last);
+        if (e != cudaSuccess) return e;
+        launch_tma2_gather(ctx, nsolve, last, ctx->g.nsteps, st);
+        return cudaGetLastError();
     }
     const size_t bytes = (size_t)nsolve * ctx->g.solve_stride * ctx->elem;
     cudaMemsetAsync(ctx->d_u0, 0, bytes, st);

@@ -442,7 +442,7 @@ cudaError_t launch_steps_strip(const oed_ctx *ctx, int nsolve, cudaStream_t st, 
         a.in = pair[pr];
         a.out = pair[pr ^ 1];
         a.m = m;
-        a.last = T == left;
+        a.last = T == left && nsteps == g.nsteps;   // (a probe's last pass stores like the others)
         e = T == 4   ? strip_pass<4>(a, ctx->strip_sms, st)
             : T == 3 ? strip_pass<3>(a, ctx->strip_sms, st)
             : T == 2 ? strip_pass<2>(a, ctx->strip_sms, st)
