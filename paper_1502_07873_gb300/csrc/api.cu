@@ -425,7 +425,7 @@ int oed_autotune(oed_ctx *ctx, int nsolve, void *stream)
     //   801x401, 3 layers: 1 solve 460 / 359 / 424, 3: 511 / 541, 56: 3366 / 5440, 200: 9287 / 18190
     //   801x401, a layer every 6 rows: 1 solve 656 / 369, 56: 8036 / 5444, 200: 24316 / 18100
     //   1301x20, 64 solves 906 / 820 / 848; 1217x9, 1 solve 386 / 328 / 310
-    // A probe takes whole passes of both; those under a millisecond are the least of three.
+    // A probe takes whole passes of both; those under 0.3 ms are the least of three.
     if (ctx->d_u2) {
         int probe = std::min(ctx->g.nsteps, std::max(nrep, 16));
         if (probe >= 4) probe = probe / 4 * 4;
@@ -439,7 +439,7 @@ int oed_autotune(oed_ctx *ctx, int nsolve, void *stream)
             };
             cudaError_t e = launch(4);   // warm
             float ms = 1e30f;
-            for (int k = 0; k < 3 && e == cudaSuccess && (k == 0 || ms < 1.0f); k++) {
+            for (int k = 0; k < 3 && e == cudaSuccess && (k == 0 || ms < 0.3f); k++) {
                 float one = 0.0f;
                 e = launch(probe);
                 if (e == cudaSuccess) e = cudaEventSynchronize(e1);
