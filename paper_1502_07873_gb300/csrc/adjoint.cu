@@ -224,16 +224,16 @@ __global__ void __launch_bounds__(128) k_adjoint64(AdjArgs<double> a, int nseg, 
     }
 }
 
-static void adjoint_step(const AdjArgs<float> &a, int nsolve, cudaStream_t st)
+static void adjoint_step(const AdjArgs<float> &a, int nsolve, int, cudaStream_t st)
 {
     const dim3 blk(32, 8, 1), grd((a.g.nx + 31) / 32, (a.g.nz + 7) / 8, nsolve);
     k_adjoint_step<float><<<grd, blk, 0, st>>>(a);
 }
 
-static void adjoint_step(const AdjArgs<double> &a, int nsolve, cudaStream_t st)
+static void adjoint_step(const AdjArgs<double> &a, int nsolve, int sms, cudaStream_t st)
 {
     constexpr int ZS = 4;   // 8 and 12 measured equal on 256 and 1000 solves of 101x76
-    const int nseg = segments64((long long)a.g.nx * nsolve, a.g.nz, ZS, 16.0, 8.0);
+    const int nseg = segments64((long long)a.g.nx * nsolve, a.g.nz, ZS, 16.0, 8.0, sms);
     const long long per = (long long)a.g.nx * nseg;
     const int most = (int)std::max(1LL, std::min((long long)nsolve, (1LL << 31) / per));   // 32-bit thread numbers
     for (int s0 = 0; s0 < nsolve; s0 += most) {
@@ -336,7 +336,7 @@ static void adjoint_impl(const oed_ctx *ctx, int nsolve, const double *y, double
         const int k = g.nsteps - m;
         a.cur = (k & 1) ? B : A;   // lambda^{m+1}
         a.nxt = (k & 1) ? A : B;   // lambda^{m+2} -> lambda^m
-        adjoint_step(a, nsolve, st);
+        adjoint_step(a, nsolve, ctx->sms, st);
         k_adjoint_post<real><<<nsolve, 128, 0, st>>>(a.nxt, w, ctx->d_rec, (const SourceDesc<real> *)ctx->d_src,
                                                      ctx->d_theta, acc, g, m);
     }

@@ -137,7 +137,8 @@ struct oed_ctx {
     oed::StepTuning tune{4, 4, 0};
     int jac_mode = OED_JAC_PAIRS;   // Jacobian form of oed_hessian
     int tma_ctas = 0;               // persistent grid of the TMA streaming kernel
-    int strip_sms = 0;              // SMs of the device, set once the multi-step kernel can run
+    int sms = 1;                    // SMs of the device
+    int strip_sms = 0;              // the same, set once the multi-step kernel can run
     int tma2_ctas = 0;              // persistent grid of the two-step TMA kernel
     // host-path staging
     cudaStream_t own_stream = nullptr;
@@ -176,7 +177,7 @@ void launch_step_probe(const oed_ctx *ctx, int nsolve, int nrep, cudaStream_t st
 
 void launch_fill_probe(const oed_ctx *ctx, int nsolve, cudaStream_t st);
 
-int segments64(long long columns, int nz, int zs, double per, double once);   // FP64 row segments
+int segments64(long long columns, int nz, int zs, double per, double once, int sms);   // FP64 row segments
 
 // stream_tma.cu
 bool tma_supported(const oed_ctx *ctx);

@@ -495,7 +495,7 @@ void launch_sources(const oed_ctx *ctx, const double *theta_nodes, int nnode, in
     for (int j = 0; j < kNT; j++) st.d[j] = step ? step[j] : 0.0;
     if (nnode <= 0) return;
     // few nodes: their time steps are spread over several blocks
-    const int parts = std::max(1, std::min((ctx->g.nsteps + 127) / 128, 304 / nnode));
+    const int parts = std::max(1, std::min((ctx->g.nsteps + 127) / 128, 2 * ctx->sms / nnode));
     const dim3 grid(nnode, parts);
     if (ctx->precision == OED_FP64)
         k_sources<double><<<grid, 128, 0, s>>>(theta_nodes, per_node, sens, ctx->stf, st, ctx->g,

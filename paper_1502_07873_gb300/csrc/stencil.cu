@@ -280,14 +280,15 @@ __global__ void k_gather(const real *__restrict__ cur, real *__restrict__ trace,
 // segment length on average.  Counted in whole rounds and without the latency it was 8% and up to
 // 39%: 15 solves of 81x41 482 us for 60 steps against 370 in one-row segments.  These have a kernel
 // without the divisions of the general one (ZS = 1; one solve of 201x101 318 -> 298 us).
-int segments64(long long columns, int nz, int zs, double per, double once)
+int segments64(long long columns, int nz, int zs, double per, double once, int sms)
 {
-    constexpr double kPipes = 4 * 152, kLatency = 8.0;
+    constexpr double kLatency = 8.0;
+    const double pipes = 4.0 * sms;
     int best = (nz + zs - 1) / zs;
     double least = 0.0;
     for (int r = zs; r >= 1; r--) {
         const int nseg = (nz + r - 1) / r, rows = (nz + nseg - 1) / nseg;
-        const double warps = (double)columns * nseg / 32.0 / kPipes;
+        const double warps = (double)columns * nseg / 32.0 / pipes;
         const double cost = std::max(1.0, 0.5 * (warps + std::ceil(warps))) * (per * rows + once) + kLatency * rows;
         if (r == zs || cost < least) {
             least = cost;
@@ -304,7 +305,7 @@ static void launch_one(const oed_ctx *ctx, int nsolve, const StepArgs<real> &a, 
     const Geometry &g = ctx->g;
     const int wz = ctx->tune.wz;
     if constexpr (sizeof(real) == 8) {
-        const int npair = (g.nx + 1) / 2, nseg = segments64((long long)npair * nsolve, g.nz, ZS, 23.0, 10.0);
+        const int npair = (g.nx + 1) / 2, nseg = segments64((long long)npair * nsolve, g.nz, ZS, 23.0, 10.0, ctx->sms);
         const long long per = (long long)npair * nseg;
         // 32-bit thread numbers: a batch past them goes in several launches
         const int most = (int)std::max(1LL, std::min((long long)nsolve, (1LL << 31) / per));
