@@ -245,7 +245,6 @@ int oed_create(oed_ctx **out, const oed_problem *p, int max_solves)
     ctx->max_solves = max_solves;
     cudaGetDevice(&ctx->device);
     cudaDeviceGetAttribute(&ctx->sms, cudaDevAttrMultiProcessorCount, ctx->device);
-    cudaDeviceGetAttribute(&ctx->sms, cudaDevAttrMultiProcessorCount, ctx->device);
     ctx->z_top.assign(p->z_top, p->z_top + p->nlayers);
     ctx->vp.assign(p->vp, p->vp + p->nlayers);
     ctx->vs.assign(p->vs, p->vs + p->nlayers);
