@@ -218,7 +218,8 @@ int run_request(oed_server *srv, Request &rq, oed_ctx *ctx, cudaStream_t st, Ent
     int *d_bad = (int *)(d_eig + 1);
     int rc = oed_set_jacobian(ctx, rq.jacobian);
     if (!rc) {
-        const auto key = std::make_tuple(rq.p.nx, rq.p.nz, rq.p.nlayers, rq.p.precision, rq.jacobian);
+        // (media of many layers, with an interface every few rows, have another fastest kernel)
+        const auto key = std::make_tuple(rq.p.nx, rq.p.nz, rq.p.nlayers / 8, rq.p.precision, rq.jacobian);
         std::tuple<int, int, int> tune;
         bool have = false;
         {
