@@ -98,3 +98,11 @@ def test_refused(P, nx, nz, prec):
     with pytest.raises(P.OedError):
         ctx.set_tuning(-3, 4, 4)
     ctx.close()
+
+
+def test_large_batches_take_the_strip_kernel(P):
+    """Without a probe, so that other work on the device cannot change the choice."""
+    w = W.tiny(nx=801, nz=401, h=2.5, nsteps=8, nrec=4, layers=W.THREE_LAYER)
+    ctx = P.Context(P.problem_from_workload(w, P.OED_FP32), max_solves=14)
+    assert ctx.autotune(14)[0] == -2
+    ctx.close()
