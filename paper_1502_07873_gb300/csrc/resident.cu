@@ -34,7 +34,7 @@
 // time function: the wavefield never leaves the chip, so this kernel is bound by the
 // shared-memory pipe (eight 64-bit accesses per column pair, row and step) and the per-step
 // barrier, not by HBM.  Large launches: 81x41 867 Gcell-upd/s (three CTAs an SM), 101x76, two
-// layers, 722, 151x76, three layers, 784, 201x101 706, 401x201 692 (clusters of six: 138 of 152 SMs
+// layers, 722, 151x76, three layers, 784, 201x101 706, 401x201 696 (clusters of six: 138 of 152 SMs
 // have a CTA).
 #include <algorithm>
 #include <cmath>

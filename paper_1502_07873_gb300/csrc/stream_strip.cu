@@ -25,8 +25,10 @@
 // What bounds it: HBM, with T = 4 at 8 B per cell-update (801x401, three layers, 672
 // solves: 705 Gcell-upd/s, 83% of the measured copy rate; 70 solves of 1601x801: 730), and
 // with few solves the blocks that do not fill the chip evenly (56 solves: 559; 7 of
-// 1601x801: 535).  The tile kernel it replaces, two steps per pass through shared memory,
-// ran these at 362, 340 and 325.  T = 2 (16 B) 390, T = 3 560: two more steps of registers
+// 1601x801: 535).  The two-step tile kernel runs these at 362, 340 and 325; it keeps the cases
+// that this one is slower on: one or two solves, whose passes wait for the longest band,
+// media with an interface every few rows (the general body takes about three times the
+// plain one's time a row) and grids of few rows (stream_tma2.cu; oed_autotune chooses).  T = 2 (16 B) 390, T = 3 560: two more steps of registers
 // cost less than their bytes.  Eight warps an SM at up to 255 registers: twelve at 168
 // spill (673 on the 672 solves), sixteen much more (360).
 #include <cmath>
@@ -393,9 +395,9 @@ static cudaError_t strip_pass(StripArgs a, int nsm, cudaStream_t st)
     // more (2 T rows computed twice, its start).  Blocks run in waves of the warps that the chip
     // holds; the last, partly filled one costs as much as the others.  A fit to 1 to 16 bands on
     // nine batches (801x401, 1601x801, 701x351, 501x501; 7 to 105 solves): the rule's choice is
-    // 0.2% slower than the best on average.  With a wave's cost spread over its blocks, Gcell-upd/s:
-    // 28 solves of 801x401 443 -> 475, 49 of 701x351 492 -> 513, 56 of 801x401 543 -> 554, 7 of
-    // 1601x801 519 -> 526.
+    // 0.2% slower than the best on average.  Against a wave's cost spread over its blocks, Gcell-upd/s:
+    // 28 solves of 801x401 443 -> 476, 49 of 701x351 492 -> 512, 56 of 801x401 543 -> 559, 7 of
+    // 1601x801 519 -> 535.
     const double strips = (double)a.nsolve * a.nstrip;
     double best = 0.0;
     for (int nb = 1; nb <= 64 && a.g.nz / nb >= 4 * T; nb++) {
