@@ -345,7 +345,8 @@ void scratch_trim()
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev >= kMaxDevices) return;
     std::lock_guard<std::mutex> lock(g_scratch_mu);
-    if (g_scratch[dev]) cudaMemPoolTrimTo(g_scratch[dev], 0);
+    if (g_scratch[dev] && cudaMemPoolTrimTo(g_scratch[dev], 0) != cudaSuccess)
+        cudaGetLastError();   // (nothing for a later call to report)
 }
 
 }  // namespace oed
