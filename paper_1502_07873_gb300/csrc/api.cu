@@ -429,7 +429,7 @@ int oed_autotune(oed_ctx *ctx, int nsolve, void *stream)
     // Where the strip kernel is ahead by half and more (over 4e6 nodes in the batch, under a quarter of
     // the rows within reach of the surface, the bottom or an interface) it is taken without a probe, so
     // that work of others on the device cannot make it look slower.  Elsewhere both are probed in turn,
-    // whole passes, the least of three rounds.
+    // 32 steps, the least of three rounds.
     if (ctx->d_u2) {
         int faces = 0;   // rows that start another layer
         for (int j = 1, l = 0; j < ctx->g.nz; j++) {
@@ -440,7 +440,7 @@ int oed_autotune(oed_ctx *ctx, int nsolve, void *stream)
         }
         const bool strip = strip_prepare(ctx) > 0, step2 = tma_supported(ctx) && tma2_prepare(ctx) > 0;
         const bool many = strip && cells > 4e6 && 9 * (faces + 2) < ctx->g.nz / 4;
-        int probe = std::min(ctx->g.nsteps, std::max(nrep, 16));
+        int probe = std::min(ctx->g.nsteps, 32);
         if (probe >= 4) probe = probe / 4 * 4;
         float least[2] = {1e30f, 1e30f};
         for (int k = 0; k < (many ? 1 : 4); k++)   // round 0 loads the code
